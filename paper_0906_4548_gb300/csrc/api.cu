@@ -702,12 +702,16 @@ class Engine : public EngineBase {
           prof.run_it(KK_X_HESSIAN, 0, sure * 7 * SB, stream,
                       [&] { launch_xy_hessian<T, N>(spec_in(it), fs(s6, 6), kp, tw, stream, sk); });
         } else {
-          prof.run_it(KK_X_HESSIAN, 0, sure * 7 * SB, stream, [&] {
+          // the relaxation writes spec_out later, so the passes' small auxiliary arrays live there
+          V* aux = spec_out(it);
+          prof.run_it(KK_X_HESSIAN, 0, sure * 4 * SB, stream, [&] {
             launch_fft_x_op<T, N>(XOP_HESSIAN, spec_in(it), nullptr, fs(s6, 6), 0, kp, nullptr, 0, 0, 0, tw, stream,
-                                  sk);
+                                  sk, aux);
           });
-          prof.run_it(KK_Y, 0, sure * 12 * SB, stream,
-                      [&] { launch_fft_y<T, N>(fs(s6, 6), 6, true, tw, stream, sk, y_threads); });
+          prof.run_it(KK_Y, 0, sure * 9 * SB, stream, [&] {
+            const YHessArgs<T> ya{{s6[0], s6[1], s6[2], s6[3], s6[4], s6[5]}, aux, sk};
+            launch_y_hessian<T, N>(&ya, 1, tw, stream);
+          });
         }
         prof.run_it(KK_RELAX, 0, sure * (7 * SB + 3 * RB), stream, [&] {
           if constexpr (sizeof(T) == 4)
@@ -732,8 +736,8 @@ class Engine : public EngineBase {
         return DGP_OK;
       };
       auto credit = [&](int iters, int yfwd) {
-        prof.credit(KK_X_HESSIAN, 7 * SB * iters);
-        prof.credit(KK_Y, (xy ? 0.0 : 12 * SB * iters) + (2 * SB + 32.0 * fblocks) * yfwd);
+        prof.credit(KK_X_HESSIAN, (xy ? 7 : 4) * SB * iters);
+        prof.credit(KK_Y, (xy ? 0.0 : 9 * SB * iters) + (2 * SB + 32.0 * fblocks) * yfwd);
         prof.credit(KK_RELAX, (7 * SB + 3 * RB) * iters);
       };
 
@@ -1134,7 +1138,7 @@ class Engine : public EngineBase {
         Engine* e = S[k];
         if ((e->wcur < 0) != (lin == 1)) continue;
         j0[k] = lin ? 0 : e->wcur;
-        xr[m] = XReal<T>{e->sDelta, nullptr, fs(e->s6, lin ? 2 : 1), 0, kp[k], nullptr};
+        xr[m] = XReal<T>{e->sDelta, nullptr, fs(e->s6, lin ? 2 : 1), 0, kp[k], nullptr, nullptr};
         fi[m] = fs(e->s6, lin ? 2 : 1);
         T* outs[2] = {e->rS, e->rD[j0[k]]};
         for (int i = 0; i < kMaxFields; ++i) fo[m].p[i] = i < (lin ? 2 : 1) ? reinterpret_cast<V*>(outs[i]) : nullptr;
@@ -1207,16 +1211,15 @@ class Engine : public EngineBase {
         Engine* e = S[k];
         const int ib = in_buf(k, it), ob = out_buf(k, it);
         sk[i] = control ? &e->d_ctl->done : nullptr;
-        xr[i] = XReal<T>{spec_in(k, it), nullptr, fs(e->s6, 6), 0, kp[k], sk[i]};
+        xr[i] = XReal<T>{spec_in(k, it), nullptr, fs(e->s6, 6), 0, kp[k], sk[i], spec_out(k, it)};
         f6[i] = fs(e->s6, 6);
-        ra[i].map[0] = e->rmaps.map[0];
         for (int q = 0; q < 6; ++q) ra[i].map[q] = e->rmaps.map[q];
         ra[i].D = e->rD[ib];
         ra[i].dsum = e->d_rstats + 4 * ib + 1;
         ra[i].S = e->rS;
         ra[i].Dnew = e->rD[ob];
-        ra[i].Snew = spec_out(k, it);
         ra[i].partials = e->partials;
+        ra[i].Snew = spec_out(k, it);
         ra[i].rp = rp[k];
         ra[i].skip = sk[i];
         ra[i].fault = &e->d_ctl->fault;
@@ -1247,8 +1250,14 @@ class Engine : public EngineBase {
       if (e0->xy_ok && e0->xy_on) {
         pf.run(KK_X_HESSIAN, 7.0 * m * SB, st, [&] { launch_xy_hessian_batch<T, N>(xr, m, tw, st); });
       } else {
-        pf.run(KK_X_HESSIAN, 7.0 * m * SB, st, [&] { launch_fft_x_batch<T, N>(XOP_HESSIAN, xr, m, tw, st); });
-        pf.run(KK_Y, 12.0 * m * SB, st, [&] { launch_fft_y_batch<T, N>(f6, sk, nullptr, m, 6, true, tw, st, yt); });
+        YHessArgs<T> ya[kBatchMax];
+        for (int i = 0; i < m; ++i) {
+          for (int q = 0; q < 6; ++q) ya[i].f[q] = f6[i].p[q];
+          ya[i].aux = xr[i].aux;
+          ya[i].skip = sk[i];
+        }
+        pf.run(KK_X_HESSIAN, 4.0 * m * SB, st, [&] { launch_fft_x_batch<T, N>(XOP_HESSIAN, xr, m, tw, st); });
+        pf.run(KK_Y, 9.0 * m * SB, st, [&] { launch_y_hessian<T, N>(ya, m, tw, st); });
       }
       pf.run(KK_RELAX, m * (7 * SB + 3 * RB), st, [&] { launch_relax_tma_batch<N>(e0->arith_mode(), ra, m, tw, st); });
       if (control) {
@@ -1395,7 +1404,7 @@ class Engine : public EngineBase {
       FieldSet<T> fi[kBatchMax], fo[kBatchMax];
       for (int k = 0; k < n; ++k) {
         Engine* e = S[k];
-        xr[k] = XReal<T>{e->sDelta, sDphi[k], fs(e->s6, 4), 14, kp[k], nullptr};
+        xr[k] = XReal<T>{e->sDelta, sDphi[k], fs(e->s6, 4), 14, kp[k], nullptr, nullptr};
         V* sp[3] = {e->s6[1], e->s6[2], e->s6[3]};
         fi[k] = fs(sp, 3);
         T* outs[3] = {e->rG[0], e->rG[1], e->rG[2]};
@@ -1648,7 +1657,7 @@ class Engine : public EngineBase {
              [&] { launch_fft_x_adj<T, N>(XOP_ADJ_PHI, in, mask, fs(s6, 2), kp, tw, stream); });
     T* ga[2] = {aG, aA};
     if ((rc = inverse_yz(s6, ga, 2))) return rc;
-    // real Hessian fields of the accepted D: H_xx, H_yy, H_xy, H_xz, H_yz (and N)
+    // real Hessian fields of the accepted D: H_yy, H_zz, H_xy, H_xz, H_yz (and N)
     if ((rc = forward_zy(rD[wcur], sD2, none))) return rc;
     RcDeriv rd{};
     if (rcbar) {
@@ -1663,10 +1672,15 @@ class Engine : public EngineBase {
                [&] { launch_finalize(pk_partials, pk_blocks, 1, d_adj + 6, stream); });
       DGP_CHECK_LAUNCH();
     }
-    prof.run(KK_X_HESSIAN, 7 * SB, stream, [&] {
-      launch_fft_x_op<T, N>(XOP_HESSIAN, sD2, nullptr, fs(s6, 6), 0, kp, nullptr, 0, 0, 0, tw, stream);
+    prof.run(KK_X_HESSIAN, 4 * SB, stream, [&] {
+      launch_fft_x_op<T, N>(XOP_HESSIAN, sD2, nullptr, fs(s6, 6), 0, kp, nullptr, 0, 0, 0, tw, stream, nullptr, sD);
     });
-    if ((rc = inverse_yz(s6, rH, 6))) return rc;
+    prof.run(KK_Y, 9 * SB, stream, [&] {
+      const YHessArgs<T> ya{{s6[0], s6[1], s6[2], s6[3], s6[4], s6[5]}, sD, nullptr};
+      launch_y_hessian<T, N>(&ya, 1, tw, stream);
+    });
+    prof.run(KK_Z_C2R, (RB + SB) * 6, stream, [&] { launch_fft_z_c2r<T, N>(fs(s6, 6), rH, 6, tw, stream); });
+    DGP_CHECK_LAUNCH();
     const double* dsum = d_rstats + 4 * wcur + 1;
     const double alpha = c.alpha, w = p.w;
     prof.run(KK_REDUCE, RB, stream,

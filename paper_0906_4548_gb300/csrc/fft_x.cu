@@ -9,10 +9,11 @@
 // transposed through shared memory once and finished over k1.
 //
 // Operations (all multipliers real-even or i*odd, so outputs stay Hermitian):
-//  HESSIAN    D(k) -> (k_i k_j / k^2) D(k) for xx, yy, xy, xz, yz and
-//             N(k) = -D(k) / kbar   (Sec. III.B: nabla_ij C(k) = -k_i k_j C(k);
-//             sqrt(-lapbar) C = kbar C = -D / kbar).  Off-diagonal pairs with a
-//             component on its Nyquist index use |k_i k_j| / k^2.
+//  HESSIAN    D(k) -> D / k^2, k_x D / k^2 and N(k) = -D(k) / kbar (Sec. III.B:
+//             nabla_ij C(k) = -k_i k_j C(k); sqrt(-lapbar) C = kbar C = -D / kbar),
+//             from which the y pass (y_hessian.cu) forms the second derivatives:
+//             the y and z wavenumbers commute with the x inverse, so three
+//             spectra leave this pass instead of six.
 //  SOURCE     S(k) = s (1 - beta / kbar) delta(k)        (RHS of Eq. FullDGP2)
 //  SOURCE_LIN S(k) and D_lin(k) = S(k) / (alpha - c2 / kbar)  (Sec. III.B)
 //  PHI_FORCE  phi(k) from Eq. FullDGP1 (or Eq. LinearDGP / GRPoisson) and
@@ -52,6 +53,7 @@ template <typename T> struct XArgs {
   int nbins;
   double shell_lo, shell_hi;
   const int* skip;
+  vec2_t<T>* aux;  // XOP_HESSIAN: the Nyquist coefficients (HessAux)
   FieldSet<T> in;  // adjoint ops: input spectra
   int in_mask;
   RcDeriv rc;      // XOP_RC: derivatives of the coefficients in r_c H0
@@ -82,9 +84,10 @@ __device__ __forceinline__ void x_forward(const vec2_t<T>* __restrict__ in, int 
 
 // trailing: end with a barrier so the next call may reuse s_T; callers that alternate
 // two transpose buffers between consecutive calls pass false.
-template <typename T, int N, bool trailing = true>
-__device__ __forceinline__ void x_inverse(vec2_t<T> (&Y)[Split<N>::N2], vec2_t<T>* __restrict__ out, int kz,
-                                          int ky0, int lane, int yl, vec2_t<T>* s_T, const vec2_t<T>* s_tw) {
+// store(x, v) receives each transformed value of the thread's column.
+template <typename T, int N, bool trailing, class Store>
+__device__ __forceinline__ void x_inverse_to(vec2_t<T> (&Y)[Split<N>::N2], int lane, int yl, vec2_t<T>* s_T,
+                                             const vec2_t<T>* s_tw, Store store) {
   using V = vec2_t<T>;
   constexpr int N1 = Split<N>::N1, N2 = Split<N>::N2, TY = XGeom<T, N>::TY;
   conj_regs(Y);
@@ -98,11 +101,17 @@ __device__ __forceinline__ void x_inverse(vec2_t<T> (&Y)[Split<N>::N2], vec2_t<T
 #pragma unroll
     for (int k1 = 0; k1 < N1; ++k1) w[k1] = s_T[(lane * N1 + k1) * TY + yl];
     dft_regs<N1, N / N1>(w, s_tw);
-    V* plane = out + (int64_t)kz * N * N;
 #pragma unroll
-    for (int m2 = 0; m2 < N1; ++m2) plane[(int64_t)(lane + N2 * m2) * N + ky0 + yl] = cconj(w[m2]);
+    for (int m2 = 0; m2 < N1; ++m2) store(lane + N2 * m2, cconj(w[m2]));
   }
   if (trailing) __syncthreads();
+}
+template <typename T, int N, bool trailing = true>
+__device__ __forceinline__ void x_inverse(vec2_t<T> (&Y)[Split<N>::N2], vec2_t<T>* __restrict__ out, int kz,
+                                          int ky0, int lane, int yl, vec2_t<T>* s_T, const vec2_t<T>* s_tw) {
+  vec2_t<T>* plane = out + (int64_t)kz * N * N;
+  x_inverse_to<T, N, trailing>(Y, lane, yl, s_T, s_tw,
+                               [&](int x, vec2_t<T> v) { plane[(int64_t)x * N + ky0 + yl] = v; });
 }
 
 // A coefficient in the element type: the host-rounded float for FP32 data, the double otherwise.
@@ -169,6 +178,41 @@ __device__ __forceinline__ void hessian_output(const vec2_t<T> (&X)[Split<N>::N2
     if (nyq) prod = fabs(prod);
     Y[k2] = cscale(X[k2], prod);
   }
+}
+
+// Output o of the split Hessian pass from the prescaled spectrum: D / k^2, k_x D / k^2 (k_x = +N/2
+// on its Nyquist index), N, and |k_x| D / k^2 (where the Nyquist rules need it).
+template <typename T, int N>
+__device__ __forceinline__ void split_output(const vec2_t<T> (&X)[Split<N>::N2], int o, int lane, T nyz2, T ikf,
+                                             vec2_t<T> (&Y)[Split<N>::N2]) {
+  constexpr int N1 = Split<N>::N1, N2 = Split<N>::N2;
+  if (o == 0) {
+#pragma unroll
+    for (int k2 = 0; k2 < N2; ++k2) Y[k2] = X[k2];
+  } else if (o == 2) {
+#pragma unroll
+    for (int k2 = 0; k2 < N2; ++k2) {
+      const T fx = (T)(float)signed_index(lane + N1 * k2, N);
+      Y[k2] = cscale(X[k2], -sqrt(fx * fx + nyz2) * ikf);
+    }
+  } else {
+#pragma unroll
+    for (int k2 = 0; k2 < N2; ++k2) {
+      const int kx = lane + N1 * k2;
+      const float fx = (float)signed_index(kx, N);
+      Y[k2] = cscale(X[k2], (T)((o == 3 || kx == N / 2) ? fabsf(fx) : fx));
+    }
+  }
+}
+// where output o goes (the buffers of H_yz, H_xz and N, see kernels.cuh); the last output only for
+// the CTAs whose plane or columns hold a Nyquist index
+template <typename T> __device__ __forceinline__ vec2_t<T>* split_dst(const FieldSet<T>& out, int o) {
+  return out.p[o == 0 ? 4 : o == 1 ? 3 : 5];
+}
+template <typename T, int N>
+__device__ __forceinline__ void split_store_abs(vec2_t<T>* aux, int kz, int ky, int x, vec2_t<T> v) {
+  if (ky == N / 2) aux[HessAux<N>::ky_nyq + (int64_t)kz * N + x] = v;
+  if (kz == N / 2) aux[HessAux<N>::kz_nyq + (int64_t)x * N + ky] = v;
 }
 
 template <typename T, int RB> struct XBatch {
@@ -441,16 +485,24 @@ __global__ void __launch_bounds__(XGeom<T, N>::THREADS, XGeom<T, N>::MIN_BLOCKS)
     return;
   }
 
-  if (OP == XOP_HESSIAN) {
+  if constexpr (OP == XOP_HESSIAN) {
     const T fy = (T)ny, fz = (T)nz;
+    const T nyz2 = fy * fy + fz * fz;
     hessian_prescale<T, N>(X0, lane, fy, fz, inv_m);
+    constexpr int NYQ1 = (N / 2) % N1, NYQ2 = (N / 2) / N1;  // k_x = N/2 in lane NYQ1's slot NYQ2
+    if (lane == NYQ1) args.aux[HessAux<N>::kx_nyq + (int64_t)kz * N + ky] = cscale(X0[NYQ2], (T)(N / 2));
     const T ikf = kp.local_only ? (T)0 : (T)1 / kc<T>(kp.kbar_fac * 2.0 * M_PI / kp.box, kp.kbkf_f);
+    const bool need_abs = kz == N / 2 || (ky0 <= N / 2 && N / 2 < ky0 + TY);
 #pragma unroll 1
-    for (int o = 0; o < 6; ++o) {
+    for (int o = 0; o < (need_abs ? 4 : 3); ++o) {
       V Y[N2];
-      hessian_output<T, N>(X0, o, lane, fy, fz, nyq_y, nyq_z, ikf, Y);
+      split_output<T, N>(X0, o, lane, nyz2, ikf, Y);
       // the outputs alternate between two transpose buffers: one barrier per output
-      x_inverse<T, N, false>(Y, args.out.p[o], kz, ky0, lane, yl, (o & 1) ? s_T2 : s_T, s_tw);
+      V* plane = split_dst(args.out, o) + (int64_t)kz * N * N + ky;
+      x_inverse_to<T, N, false>(Y, lane, yl, (o & 1) ? s_T2 : s_T, s_tw, [&](int x, V v) {
+        if (o < 3) plane[(int64_t)x * N] = v;
+        else split_store_abs<T, N>(args.aux, kz, ky, x, v);
+      });
     }
     return;
   }
@@ -553,8 +605,7 @@ __global__ void __launch_bounds__(XGeom<T, N>::THREADS, XGeom<T, N>::MIN_BLOCKS)
   }
 
   int nout;
-  if (OP == XOP_HESSIAN) nout = 6;
-  else if (OP == XOP_SOURCE) nout = 1;
+  if (OP == XOP_SOURCE) nout = 1;
   else if (OP == XOP_SOURCE_LIN || OP == XOP_SHELL) nout = 2;
   else nout = 4;
   for (int o = 0; o < nout; ++o) {
@@ -571,18 +622,7 @@ __global__ void __launch_bounds__(XGeom<T, N>::THREADS, XGeom<T, N>::MIN_BLOCKS)
         const T inv_n2 = s_inv[k2 * NT + threadIdx.x];
         // 1 / kbar = 1 / (kbar_fac * kf * |n|)
         const T ikb = s_ikb[k2 * NT + threadIdx.x];
-        if (OP == XOP_HESSIAN) {
-          T m;
-          switch (o) {
-            case 0: m = (T)(nx * nx) * inv_n2; break;
-            case 1: m = (T)(ny * ny) * inv_n2; break;
-            case 2: m = (T)((nyq_x || nyq_y) ? abs(nx * ny) : nx * ny) * inv_n2; break;
-            case 3: m = (T)((nyq_x || nyq_z) ? abs(nx * nz) : nx * nz) * inv_n2; break;
-            case 4: m = (T)((nyq_y || nyq_z) ? abs(ny * nz) : ny * nz) * inv_n2; break;
-            default: m = -ikb; break;
-          }
-          r = cscale(X0[k2], m * inv_m);
-        } else if (OP == XOP_SOURCE || OP == XOP_SOURCE_LIN) {
+        if (OP == XOP_SOURCE || OP == XOP_SOURCE_LIN) {
           const T sfac = kc<T>(kp.s, kp.s_f) * ((T)1 - kc<T>(kp.beta, kp.beta_f) * ikb) * inv_m;
           r = cscale(X0[k2], sfac);
           if (o == 1) r = cscale(r, (T)1 / (kc<T>(kp.alpha, kp.alpha_f) - kc<T>(kp.c2, kp.c2_f) * ikb));
@@ -635,11 +675,11 @@ __global__ void __launch_bounds__(XGeom<T, N>::THREADS, XGeom<T, N>::MIN_BLOCKS)
 // transposes and the stores).
 template <int N> struct XSGeom {
   static constexpr int N1 = Split<N>::N1, N2 = Split<N>::N2;
-  static constexpr int TY = 16 < N ? 16 : N;
+  static constexpr int TY = 16;
   static constexpr int THREADS = TY * N1;
   static constexpr int TILE = N * TY;  // complex
-  static constexpr size_t SMEM = sizeof(float2) * ((size_t)kTwiddleTables * N + 2 * (size_t)TILE);
-  static constexpr int MINB = THREADS <= 256 ? 3 : 1;
+  static constexpr size_t SMEM = sizeof(float2) * ((size_t)N + 2 * (size_t)TILE);  // phase table, two tiles
+    static constexpr int MINB = THREADS >= 128 ? 768 / THREADS : 6;
 };
 
 template <int N, int RB>
@@ -652,16 +692,15 @@ __global__ void __launch_bounds__(XSGeom<N>::THREADS, XSGeom<N>::MINB)
   if (args.skip && *args.skip) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   V* s_tw = reinterpret_cast<V*>(smem_raw);
-  V* A = s_tw + kTwiddleTables * N;  // the spectrum, rows in digit order
+  V* A = s_tw + N;  // the spectrum, rows in digit order
   V* B = A + G::TILE;                // one output at a time
-  load_twiddles(s_tw, g_tw, N);
   const int tid = threadIdx.x;
+  for (int i = tid; i < N; i += G::THREADS) s_tw[i] = g_tw[N + i];
   const int yl = tid % TY, q = tid / TY;  // q: j2 / n2 (stages 1 and 4) or k1 (stages 2 and 3)
   const int kz = blockIdx.y, ky0 = blockIdx.x * TY, ky = ky0 + yl;
   const int nz = kz == N / 2 ? -(N / 2) : kz;
-  const bool nyq_y = ky == N / 2, nyq_z = kz == N / 2;
   const KParams& kp = args.kp;
-  const float fy = (float)signed_index(ky, N), fz = (float)nz;
+  const float fy = (float)signed_index(ky, N), fz = (float)nz, nyz2 = fy * fy + fz * fz;
   const bool st14 = q < N2;  // stages over N1 points: TY x N2 tasks
   __syncthreads();
   // forward, stage 1: x = N2 j1 + j2 from global, transform over j1, twiddle, rows N2 k1 + j2
@@ -672,7 +711,7 @@ __global__ void __launch_bounds__(XSGeom<N>::THREADS, XSGeom<N>::MINB)
     for (int j1 = 0; j1 < N1; ++j1) v[j1] = plane[(int64_t)(N2 * j1 + q) * N + ky];
     dft_regs<N1, N / N1>(v, s_tw);
 #pragma unroll
-    for (int k1 = 0; k1 < N1; ++k1) A[(N2 * k1 + q) * TY + yl] = k1 == 0 ? v[k1] : cmul(v[k1], s_tw[N + k1 * N2 + q]);
+    for (int k1 = 0; k1 < N1; ++k1) A[(N2 * k1 + q) * TY + yl] = k1 == 0 ? v[k1] : cmul(v[k1], s_tw[k1 * N2 + q]);
   }
   __syncthreads();
   // forward, stage 2 (k1 = q): transform over j2; X[k1 + N1 k2] to row N2 k1 + k2, prescaled
@@ -682,23 +721,26 @@ __global__ void __launch_bounds__(XSGeom<N>::THREADS, XSGeom<N>::MINB)
     for (int j2 = 0; j2 < N2; ++j2) X[j2] = A[(N2 * q + j2) * TY + yl];
     dft_regs<N2, N / N2>(X, s_tw);
     hessian_prescale<float, N>(X, q, fy, fz, kp.inv_m_f);
+    constexpr int NYQ1 = (N / 2) % N1, NYQ2 = (N / 2) / N1;  // k_x = N/2 in slot NYQ2 of k1 = NYQ1
+    if (q == NYQ1) args.aux[HessAux<N>::kx_nyq + (int64_t)kz * N + ky] = cscale(X[NYQ2], (float)(N / 2));
 #pragma unroll
     for (int k2 = 0; k2 < N2; ++k2) A[(N2 * q + k2) * TY + yl] = X[k2];
   }
   __syncthreads();
   const float ikf = kp.local_only ? 0.f : 1.f / kp.kbkf_f;
+  const bool need_abs = kz == N / 2 || (ky0 <= N / 2 && N / 2 < ky0 + TY);
 #pragma unroll 1
-  for (int o = 0; o < 6; ++o) {
+  for (int o = 0; o < (need_abs ? 4 : 3); ++o) {
     // inverse, stage 1 (k1 = q): multiplier as read, conj, transform over k2, twiddle
     {
       V X[N2], Y[N2];
 #pragma unroll
       for (int k2 = 0; k2 < N2; ++k2) X[k2] = A[(N2 * q + k2) * TY + yl];
-      hessian_output<float, N>(X, o, q, fy, fz, nyq_y, nyq_z, ikf, Y);
+      split_output<float, N>(X, o, q, nyz2, ikf, Y);
       conj_regs(Y);
       dft_regs<N2, N / N2>(Y, s_tw);
 #pragma unroll
-      for (int n2 = 0; n2 < N2; ++n2) B[(N2 * q + n2) * TY + yl] = n2 == 0 ? Y[n2] : cmul(Y[n2], s_tw[N + q * N2 + n2]);
+      for (int n2 = 0; n2 < N2; ++n2) B[(N2 * q + n2) * TY + yl] = n2 == 0 ? Y[n2] : cmul(Y[n2], s_tw[q * N2 + n2]);
     }
     __syncthreads();
     // inverse, stage 2 (n2 = q): transform over k1, conj, x = N2 n1 + n2 to global
@@ -707,9 +749,14 @@ __global__ void __launch_bounds__(XSGeom<N>::THREADS, XSGeom<N>::MINB)
 #pragma unroll
       for (int k1 = 0; k1 < N1; ++k1) w[k1] = B[(N2 * k1 + q) * TY + yl];
       dft_regs<N1, N / N1>(w, s_tw);
-      V* plane = args.out.p[o] + (int64_t)kz * N * N;
+      if (o < 3) {
+        V* plane = split_dst(args.out, o) + (int64_t)kz * N * N;
 #pragma unroll
-      for (int n1 = 0; n1 < N1; ++n1) plane[(int64_t)(N2 * n1 + q) * N + ky] = cconj(w[n1]);
+        for (int n1 = 0; n1 < N1; ++n1) plane[(int64_t)(N2 * n1 + q) * N + ky] = cconj(w[n1]);
+      } else {
+#pragma unroll
+        for (int n1 = 0; n1 < N1; ++n1) split_store_abs<float, N>(args.aux, kz, ky, N2 * n1 + q, cconj(w[n1]));
+      }
     }
     __syncthreads();
   }
@@ -739,15 +786,15 @@ static void launch_x(const XArgs<T>* a, int count, const vec2_t<T>* tw, cudaStre
                                                                           : sizeof(T) * 2 * Split<N>::N2 * G::THREADS);
   const size_t per_bin = PK ? sizeof(double) * NW * NBS : 0;
   const size_t smem = base + tables + per_bin * a[0].nbins;
-  raise_smem_limit<k_fft_x<T, N, OP, RB>>(base + tables + per_bin * (N / 2));
   if constexpr (OP == XOP_HESSIAN && sizeof(T) == 4 && N <= 256) {
     launch_xs<N, RB>(a, count, tw, s);  // the shared-memory version of the same pass
-    return;
+  } else {
+    raise_smem_limit<k_fft_x<T, N, OP, RB>>(base + tables + per_bin * (N / 2));
+    XBatch<T, RB> xb;
+    for (int r = 0; r < count; ++r) xb.a[r] = a[r];
+    dim3 grid(N / G::TY, N / 2 + 1, count);
+    k_fft_x<T, N, OP, RB><<<grid, G::THREADS, smem, s>>>(xb, tw);
   }
-  XBatch<T, RB> xb;
-  for (int r = 0; r < count; ++r) xb.a[r] = a[r];
-  dim3 grid(N / G::TY, N / 2 + 1, count);
-  k_fft_x<T, N, OP, RB><<<grid, G::THREADS, smem, s>>>(xb, tw);
 }
 
 template <typename T, int N>
@@ -762,6 +809,7 @@ void launch_fft_x_batch(int op, const XReal<T>* rz, int count, const vec2_t<T>* 
     a[r].nout_mask = rz[r].nout_mask;
     a[r].kp = rz[r].kp;
     a[r].skip = rz[r].skip;
+    a[r].aux = rz[r].aux;
     for (int i = 0; i < kMaxFields; ++i) a[r].in.p[i] = nullptr;
   }
   switch (op) {
@@ -776,9 +824,10 @@ void launch_fft_x_batch(int op, const XReal<T>* rz, int count, const vec2_t<T>* 
 template <typename T, int N>
 void launch_fft_x_op(int op, const vec2_t<T>* in0, const vec2_t<T>* in1, const FieldSet<T>& out, int nout_mask,
                      const KParams& kp, double* pk_partials, int nbins, double shell_lo, double shell_hi,
-                     const vec2_t<T>* tw, cudaStream_t s, const int* skip) {
+                     const vec2_t<T>* tw, cudaStream_t s, const int* skip, vec2_t<T>* aux) {
   XArgs<T> a{};
   a.skip = skip;
+  a.aux = aux;
   a.in0 = in0; a.in1 = in1; a.out = out; a.nout_mask = nout_mask; a.kp = kp;
   a.pk_partials = pk_partials; a.nbins = nbins; a.shell_lo = shell_lo; a.shell_hi = shell_hi;
   a.in_mask = 0;
@@ -1058,7 +1107,7 @@ DGP_INST_XY(512)
 #define DGP_INST_X(T, N)                                                                            \
   template void launch_fft_x_op<T, N>(int, const vec2_t<T>*, const vec2_t<T>*, const FieldSet<T>&, int, \
                                       const KParams&, double*, int, double, double, const vec2_t<T>*,   \
-                                      cudaStream_t, const int*);                                        \
+                                      cudaStream_t, const int*, vec2_t<T>*);                             \
   template void launch_fft_x_adj<T, N>(int, const FieldSet<T>&, int, const FieldSet<T>&, const KParams&,  \
                                        const vec2_t<T>*, cudaStream_t);                                  \
   template void launch_fft_x_rc<T, N>(const FieldSet<T>&, int, const KParams&, const RcDeriv&, double*,   \
@@ -1070,6 +1119,7 @@ DGP_INST_XB(16) DGP_INST_XB(32) DGP_INST_XB(48) DGP_INST_XB(64) DGP_INST_XB(96) 
   DGP_INST_X(T, 256) DGP_INST_X(T, 512) DGP_INST_X(T, 48) DGP_INST_X(T, 96)
 DGP_INST_X_ALL(float)
 DGP_INST_X_ALL(double)
+#undef DGP_INST_XB
 #define DGP_INST_XB(T) template int x_pass_blocks<T, 16>(); template int x_pass_blocks<T, 32>(); \
   template int x_pass_blocks<T, 64>(); template int x_pass_blocks<T, 128>(); \
   template int x_pass_blocks<T, 256>(); template int x_pass_blocks<T, 512>(); \

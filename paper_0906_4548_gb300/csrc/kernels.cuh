@@ -114,7 +114,8 @@ void launch_fft_z_c2r_batch(const FieldSet<T>* in, const FieldSet<T>* out, int n
 template <typename T, int N>
 void launch_fft_x_op(int op, const vec2_t<T>* in0, const vec2_t<T>* in1, const FieldSet<T>& out,
                      int nout_mask, const KParams& kp, double* pk_partials, int nbins, double shell_lo,
-                     double shell_hi, const vec2_t<T>* tw, cudaStream_t s, const int* skip = nullptr);
+                     double shell_hi, const vec2_t<T>* tw, cudaStream_t s, const int* skip = nullptr,
+                     vec2_t<T>* aux = nullptr);
 
 // Adjoint x-passes (several y-transformed input spectra):
 //  XOP_ADJ_PHI: inputs (mask bit f) phibar, gbar_x, gbar_y, gbar_z; with
@@ -141,6 +142,7 @@ template <typename T> struct XReal {
   int nout_mask;
   KParams kp;
   const int* skip;
+  vec2_t<T>* aux;  // XOP_HESSIAN: HessAux<N>::size values
 };
 template <typename T, int N>
 void launch_fft_x_batch(int op, const XReal<T>* r, int count, const vec2_t<T>* tw, cudaStream_t s);
@@ -181,7 +183,7 @@ struct RelaxMaps {
 };
 // Arguments of one realisation's relaxation pass (relax_tma.cu).
 struct RelaxTmaArgs {
-  CUtensorMap map[6];   // y-inverted spectra of H_xx, H_yy, H_xy, H_xz, H_yz, N
+  CUtensorMap map[6];   // y-inverted spectra: two of H_xx, H_yy, H_zz, then H_xy, H_xz, H_yz, N
   const float* D;       // current iterate (its mean = dsum / N^3)
   const double* dsum;
   const float* S;       // source field
@@ -199,6 +201,26 @@ template <int RB> struct RelaxTmaBatch {
 };
 template <int N>
 void launch_relax_tma_batch(int arith, const RelaxTmaArgs* a, int count, const float2* tw, cudaStream_t s);
+
+// The Hessian passes of an iteration.  The x pass (XOP_HESSIAN) leaves three spectra in the buffers
+// of outputs 4, 3 and 5 (G0 = IFFT_x[D / k^2], G1 = IFFT_x[k_x D / k^2], N) and the auxiliary
+// coefficients of the Nyquist rules in aux; the y pass (y_hessian.cu) turns them into the six
+// relaxation inputs f[0..5] = H_yy, H_zz, H_xy, H_xz, H_yz, N, transformed back along x and y.
+template <int N> struct HessAux {  // offsets (complex) into aux; aux is dead once the y pass has run
+  static constexpr int64_t kx_nyq = 0;                               // [kz][ky]: (N/2) D / k^2 at k_x = N/2
+  static constexpr int64_t ky_nyq = (int64_t)(N / 2 + 1) * N;         // [kz][x]: IFFT_x[|k_x| D / k^2] at k_y = N/2
+  static constexpr int64_t kz_nyq = 2 * (int64_t)(N / 2 + 1) * N;     // [x][ky]: the same at k_z = N/2
+  static constexpr int64_t size = kz_nyq + (int64_t)N * N;
+  static_assert(size <= (int64_t)(N / 2 + 1) * N * N, "aux fits a half spectrum");
+};
+template <typename T> struct YHessArgs {
+  vec2_t<T>* f[6];
+  const vec2_t<T>* aux;
+  const int* skip;
+};
+// count <= kBatchMax realisations of one mesh size (more than one: FP32, N <= 128)
+template <typename T, int N>
+void launch_y_hessian(const YHessArgs<T>* a, int count, const vec2_t<T>* tw, cudaStream_t s);
 
 // Plane-resident Hessian pass (plane.cu) for count <= kBatchMax realisations of one mesh size
 // n (FP32 data; plane_hessian_supported(n)): from the z spectrum in (layout S[kz][x][y]) of
@@ -232,7 +254,7 @@ void launch_sph_update(const T* S, T* D, int64_t m, double alpha, double* partia
 
 // Adjoint relaxation (J^T lam = g on mean-free fields, w-split as the forward
 // iteration).  d = D - mean(D) (mean = dsum / m), diag = 2 (1 - w) d + alpha.
-//  products: P[f m + i] = H_f lam for f = xx, yy, zz (= d - xx - yy), xy, xz, yz.
+//  products: P[f m + i] = H_f lam for f = xx (= d - yy - zz), yy, zz, xy, xz, yz, H5 = yy, zz, xy, xz, yz.
 //  update_a: u = (g - 2 w d lam - Q) / diag; partials[b][2] = (sum u, sum diag (lam - u)).
 //  update_b: sums = [sum u, sum diag (lam - u), sum 1/diag]; lam <- u + c / diag with
 //    c = -mean(u) / mean(1/diag) (lam stays mean-free); partials[b] = sum |diag (lam_old - u)

@@ -374,16 +374,16 @@ __device__ __forceinline__ T block_mean_d(const double* dsum, int64_t m) {
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_adj_products(const T* __restrict__ lam, const T* __restrict__ D,
-                                                      const double* __restrict__ dsum, const T* __restrict__ hxx,
-                                                      const T* __restrict__ hyy, const T* __restrict__ hxy,
+                                                      const double* __restrict__ dsum, const T* __restrict__ hyy,
+                                                      const T* __restrict__ hzz, const T* __restrict__ hxy,
                                                       const T* __restrict__ hxz, const T* __restrict__ hyz,
                                                       T* __restrict__ P, int64_t m) {
   const T mean = block_mean_d<T>(dsum, m);
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-    const T l = lam[i], a = hxx[i], b = hyy[i];
-    P[i] = a * l;
-    P[m + i] = b * l;
-    P[2 * m + i] = ((D[i] - mean) - a - b) * l;
+    const T l = lam[i], a = hyy[i], b = hzz[i];
+    P[i] = ((D[i] - mean) - a - b) * l;
+    P[m + i] = a * l;
+    P[2 * m + i] = b * l;
     P[3 * m + i] = hxy[i] * l;
     P[4 * m + i] = hxz[i] * l;
     P[5 * m + i] = hyz[i] * l;
