@@ -442,7 +442,8 @@ class Engine : public EngineBase {
     if (cudaMalloc(&sDelta, sb) != cudaSuccess) return DGP_E_NOMEM;
     nblocks = num_sms() * 4;
     if constexpr (sizeof(T) == 4) {
-      if (relax_maps<N>(s6, &rmaps) != 0) return DGP_E_CUDA;
+      float2* const snew[2] = {sD, sD2};
+      if (relax_maps<N>(s6, snew, &rmaps) != 0) return DGP_E_CUDA;
       fblocks = relax_tma_blocks<N>();
     } else {
       fblocks = fused_relax_blocks<T, N>();
@@ -1213,13 +1214,12 @@ class Engine : public EngineBase {
         sk[i] = control ? &e->d_ctl->done : nullptr;
         xr[i] = XReal<T>{spec_in(k, it), nullptr, fs(e->s6, 6), 0, kp[k], sk[i], spec_out(k, it)};
         f6[i] = fs(e->s6, 6);
-        for (int q = 0; q < 6; ++q) ra[i].map[q] = e->rmaps.map[q];
+        relax_set_maps(e->rmaps, spec_out(k, it), &ra[i]);
         ra[i].D = e->rD[ib];
         ra[i].dsum = e->d_rstats + 4 * ib + 1;
         ra[i].S = e->rS;
         ra[i].Dnew = e->rD[ob];
         ra[i].partials = e->partials;
-        ra[i].Snew = spec_out(k, it);
         ra[i].rp = rp[k];
         ra[i].skip = sk[i];
         ra[i].fault = &e->d_ctl->fault;

@@ -179,11 +179,14 @@ template <typename T, int N> int fused_relax_blocks();
 // to 1 and its CTA returns.  withhold (a test hook) leaves the first pair's
 // copy unissued, so that the first wait runs out.
 struct RelaxMaps {
-  CUtensorMap map[6];
+  CUtensorMap map[6];      // the six spectra read
+  CUtensorMap out_map[2];  // the two buffers the z spectrum of D_new alternates between
+  const float2* out[2];
 };
 // Arguments of one realisation's relaxation pass (relax_tma.cu).
 struct RelaxTmaArgs {
   CUtensorMap map[6];   // y-inverted spectra: two of H_xx, H_yy, H_zz, then H_xy, H_xz, H_yz, N
+  CUtensorMap out_map;  // Snew, for the passes that store it as tiles
   const float* D;       // current iterate (its mean = dsum / N^3)
   const double* dsum;
   const float* S;       // source field
@@ -239,7 +242,9 @@ void launch_plane_hessian_batch(int n, const PlaneArgs* a, int count, const floa
 // realisation r's block partials and applies its stop rules (as the control CTA of the y pass);
 // realisations whose skip flag is set are left alone.
 void launch_control_batch(const YControl* ctl, const int* const* skip, int count, cudaStream_t s);
-template <int N> int relax_maps(float2* const* spec6, RelaxMaps* out);
+template <int N> int relax_maps(float2* const* spec6, float2* const* snew2, RelaxMaps* out);
+// the tensor maps of a pass that writes Snew (one of the two buffers given to relax_maps)
+void relax_set_maps(const RelaxMaps& maps, float2* Snew, RelaxTmaArgs* a);
 template <int N> int relax_tma_blocks();
 template <int N>
 void launch_relax_tma(int arith, const RelaxMaps& maps, const float* D, const double* dsum, const float* S,

@@ -1,4 +1,6 @@
 // Fused z pass of one relaxation iteration for FP32 mesh data (Secs. III.B-C).
+// Two kernels share the host side and the arithmetic below: k_relax_rows (relax_rows.cuh) for
+// power-of-two meshes and k_relax_tma for the others.
 //
 // A CTA owns TY = 16 consecutive rows (x, y0 .. y0 + 15) of the mesh.  It
 //   1. inverse-transforms along z the six y-inverted spectra of those rows as
@@ -230,7 +232,7 @@ template <int N> struct RGeom {
   static constexpr int TW = N * 8;                        // the phase table W_N^{j2 k1}
   static constexpr int EXTRA = 64 + 4 * 32 * 8 + 32;      // mbarriers, warp partials, the mean
   static constexpr size_t SMEM = 1024 + BUF0 + BUF1 + TW + EXTRA;
-  static constexpr int MINB = THREADS <= 256 ? 3 : 1;
+    static constexpr int MINB = THREADS <= 256 ? 3 : 1;
   static_assert(2 * ROWB == 256 && TY * 8 == 128, "a tile row is one 128-byte swizzle row");
   static_assert(P * RS * 8 <= BUF0, "forward transpose fits the first buffer");
   static_assert(BUF0 % 1024 == 0 && BSTRIDE % 1024 == 0, "TMA tiles start on 1024-byte boundaries");
@@ -385,7 +387,7 @@ __global__ void __launch_bounds__(RGeom<N>::THREADS, RGeom<N>::MINB)
   using Sum = typename AR::Sum;
   constexpr int N1 = G::N1, N2 = G::N2, TY = G::TY, NK = G::NK, P = G::P, ROWP = G::ROWP;
   extern __shared__ unsigned char smem_raw[];
-  unsigned char* buf0 = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  unsigned char* buf0 = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);
   unsigned char* buf1 = buf0 + G::BUF0;
   float2* s_tw = reinterpret_cast<float2*>(buf1 + G::BUF1);
   uint64_t* bars = reinterpret_cast<uint64_t*>(s_tw + N);  // [2]
@@ -629,7 +631,20 @@ __global__ void __launch_bounds__(RGeom<N>::THREADS, RGeom<N>::MINB)
   }
 }
 
+}  // namespace dgp
+
+#include "relax_rows.cuh"
+
+namespace dgp {
+
 // ---------------------------------------------------------------- host side
+// Which version serves a mesh: rows inside warps for N a power of two (against k_relax_tma, one
+// GB300, mixed arithmetic: 64^3 12.3 -> 10.2 us, 128^3 32 -> 23.4, 256^3 160 -> 135, 512^3
+// 1937 -> 1449); k_relax_tma for 48 and 96, whose rows of 3 or 6 lanes do not fill warps.
+template <int N> constexpr bool kRowsInWarps = N != 48 && N != 96;
+template <int N, bool ROWS> struct MapBox { static constexpr int k = RGeom<N>::BOXK; };
+template <int N> struct MapBox<N, true> { static constexpr int k = RowGeom<N>::BOXK; };
+
 static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
   static PFN_cuTensorMapEncodeTiled_v12000 fn = nullptr;
   static std::once_flag once;
@@ -647,18 +662,20 @@ static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 }
 
 template <int N>
-int relax_maps(float2* const* spec6, RelaxMaps* out) {
+int relax_maps(float2* const* spec6, float2* const* snew2, RelaxMaps* out) {
   using G = RGeom<N>;
   const PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
   if (!enc) return 1;
   // the half spectrum S[kz][x][y] as floats: dim 0 = 2N floats along y, dim 1 = x, dim 2 = kz
   const cuuint64_t dims[3] = {(cuuint64_t)2 * N, (cuuint64_t)N, (cuuint64_t)G::NK};
   const cuuint64_t strides[2] = {(cuuint64_t)2 * N * 4, (cuuint64_t)N * 2 * N * 4};
-  const cuuint32_t box[3] = {(cuuint32_t)2 * G::TY, 1, (cuuint32_t)G::BOXK};
+  const cuuint32_t box[3] = {(cuuint32_t)2 * G::TY, 1, (cuuint32_t)MapBox<N, kRowsInWarps<N>>::k};
   const cuuint32_t es[3] = {1, 1, 1};
-  for (int f = 0; f < 6; ++f) {
-    const CUresult r = enc(reinterpret_cast<CUtensorMap*>(&out->map[f]), CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3,
-                           spec6[f], dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
+  out->out[0] = snew2[0];
+  out->out[1] = snew2[1];
+  for (int f = 0; f < 8; ++f) {
+    const CUresult r = enc(f < 6 ? &out->map[f] : &out->out_map[f - 6], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3,
+                           f < 6 ? spec6[f] : snew2[f - 6], dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE,
                            CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) return 1;
@@ -666,16 +683,27 @@ int relax_maps(float2* const* spec6, RelaxMaps* out) {
   return 0;
 }
 
+void relax_set_maps(const RelaxMaps& maps, float2* Snew, RelaxTmaArgs* a) {
+  memcpy(a->map, maps.map, sizeof(a->map));
+  a->out_map = maps.out_map[Snew == maps.out[0] ? 0 : 1];
+  a->Snew = Snew;
+}
+
 template <int N> int relax_tma_blocks() { return (N / RGeom<N>::TY) * N; }
 
 template <int N, class AR, int RB>
 static void launch_rt(const RelaxTmaArgs* a, int count, const float2* tw, cudaStream_t s) {
-  using G = RGeom<N>;
   RelaxTmaBatch<RB> b;
   for (int r = 0; r < count; ++r) b.a[r] = a[r];
-  raise_smem_limit<k_relax_tma<N, AR, RB>>(G::SMEM);
-  dim3 grid(N / G::TY, N, count);
-  k_relax_tma<N, AR, RB><<<grid, G::THREADS, G::SMEM, s>>>(b, tw);
+  if constexpr (kRowsInWarps<N>) {
+    using G = RowGeom<N>;
+    raise_smem_limit<k_relax_rows<N, AR, RB>>(G::SMEM);
+    k_relax_rows<N, AR, RB><<<dim3(N / G::TY, N, count), G::THREADS, G::SMEM, s>>>(b, tw);
+  } else {
+    using G = RGeom<N>;
+    raise_smem_limit<k_relax_tma<N, AR, RB>>(G::SMEM);
+    k_relax_tma<N, AR, RB><<<dim3(N / G::TY, N, count), G::THREADS, G::SMEM, s>>>(b, tw);
+  }
 }
 
 template <int N, class AR>
@@ -689,8 +717,8 @@ void launch_relax_tma(int arith, const RelaxMaps& maps, const float* D, const do
                       float* Dnew, float2* Snew, RelaxParams rp, double* partials, const float2* tw, cudaStream_t s,
                       const int* skip, int* fault, unsigned long long wait_ns, int withhold) {
   RelaxTmaArgs a;
-  memcpy(a.map, maps.map, sizeof(a.map));
-  a.D = D; a.dsum = dsum; a.S = S; a.Dnew = Dnew; a.Snew = Snew; a.partials = partials; a.rp = rp;
+  relax_set_maps(maps, Snew, &a);
+  a.D = D; a.dsum = dsum; a.S = S; a.Dnew = Dnew; a.partials = partials; a.rp = rp;
   a.skip = skip; a.fault = fault; a.wait_ns = wait_ns; a.withhold = withhold;
   launch_relax_tma_batch<N>(arith, &a, 1, tw, s);
 }
@@ -705,7 +733,7 @@ void launch_relax_tma_batch(int arith, const RelaxTmaArgs* a, int count, const f
 }
 
 #define DGP_INST_RT(N)                                                                                          \
-  template int relax_maps<N>(float2* const*, RelaxMaps*);                                                     \
+  template int relax_maps<N>(float2* const*, float2* const*, RelaxMaps*);                                                     \
   template int relax_tma_blocks<N>();                                                                         \
   template void launch_relax_tma<N>(int, const RelaxMaps&, const float*, const double*, const float*, float*,  \
                                     float2*, RelaxParams, double*, const float2*, cudaStream_t, const int*, int*, \
