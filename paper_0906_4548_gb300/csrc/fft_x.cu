@@ -667,19 +667,21 @@ __global__ void __launch_bounds__(XGeom<T, N>::THREADS, XGeom<T, N>::MIN_BLOCKS)
 // Hessian x pass for FP32 data with the spectrum in shared memory (N <= 256).
 //
 // The same work as k_fft_x's Hessian operation for one kz plane and TY ky columns, with the
-// x transforms done as in-place four-step stages on a [x][ky] tile in shared memory: the
-// forward transform leaves X[k1 + N1 k2] at row N2 k1 + k2 (digit order), and each output's
-// inverse reads that order back, forming the multiplier as it reads.  No thread holds the
-// spectrum in registers, so a thread needs about half the registers of the register-resident
-// version, and three CTAs fit on an SM instead of two (more warps to hide the latency of the
-// transposes and the stores).
+// x transforms as four-step stages through a [x][ky] tile in shared memory: the forward transform
+// leaves X[k1 + N1 k2] in digit order (row N2 k1 + k2, or the registers of thread k1), and each
+// output's inverse starts from that order, forming the multiplier as it reads.
 template <int N> struct XSGeom {
   static constexpr int N1 = Split<N>::N1, N2 = Split<N>::N2;
   static constexpr int TY = 16;
   static constexpr int THREADS = TY * N1;
   static constexpr int TILE = N * TY;  // complex
   static constexpr size_t SMEM = sizeof(float2) * ((size_t)N + 2 * (size_t)TILE);  // phase table, two tiles
-    static constexpr int MINB = THREADS >= 128 ? 768 / THREADS : 6;
+      // REG: the spectrum and the thread's phases W^{q m} stay in registers (two CTAs of 126 registers at
+  // 256^3) instead of being read from shared memory for every output; half the shared-memory
+  // instructions, which are what the pass waits for: 75 -> 67.5 us.  At 128^3 the tile version in 64
+  // registers lets all 520 CTAs run at once (15.9 us against 17.6 with REG, 17.8 with three per SM).
+  static constexpr bool REG = N != 128;
+  static constexpr int MINB = N == 128 ? 4 : THREADS < 128 ? 6 : 512 / THREADS;
 };
 
 template <int N, int RB>
@@ -688,66 +690,82 @@ __global__ void __launch_bounds__(XSGeom<N>::THREADS, XSGeom<N>::MINB)
   using G = XSGeom<N>;
   using V = float2;
   constexpr int N1 = G::N1, N2 = G::N2, TY = G::TY;
+  constexpr bool REG = G::REG;
   const XArgs<float>& args = xb.a[RB > 1 ? blockIdx.z : 0];
   if (args.skip && *args.skip) return;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  V* s_tw = reinterpret_cast<V*>(smem_raw);
-  V* A = s_tw + N;  // the spectrum, rows in digit order
-  V* B = A + G::TILE;                // one output at a time
+  V* A = reinterpret_cast<V*>(smem_raw);  // the spectrum, rows in digit order (REG: a transpose)
+  V* B = A + G::TILE;                     // one output at a time
+  V* s_tw = B + G::TILE;                  // !REG: the phase table
   const int tid = threadIdx.x;
-  for (int i = tid; i < N; i += G::THREADS) s_tw[i] = g_tw[N + i];
   const int yl = tid % TY, q = tid / TY;  // q: j2 / n2 (stages 1 and 4) or k1 (stages 2 and 3)
   const int kz = blockIdx.y, ky0 = blockIdx.x * TY, ky = ky0 + yl;
   const int nz = kz == N / 2 ? -(N / 2) : kz;
   const KParams& kp = args.kp;
   const float fy = (float)signed_index(ky, N), fz = (float)nz, nyz2 = fy * fy + fz * fz;
   const bool st14 = q < N2;  // stages over N1 points: TY x N2 tasks
-  __syncthreads();
   // forward, stage 1: x = N2 j1 + j2 from global, transform over j1, twiddle, rows N2 k1 + j2
+  V v[N1];
   if (st14) {
     const V* plane = args.in0 + (int64_t)kz * N * N;
-    V v[N1];
 #pragma unroll
     for (int j1 = 0; j1 < N1; ++j1) v[j1] = plane[(int64_t)(N2 * j1 + q) * N + ky];
+  }
+  // the thread's phases W^{q m}: the same ones serve the forward's first stage and every inverse
+  V tw[N1];
+  if constexpr (REG) {
+#pragma unroll
+    for (int m = 1; m < N1; ++m) tw[m] = g_tw[N + (m < N2 ? q * N2 + m : m * N2 + (st14 ? q : 0))];
+  } else {
+    for (int i = tid; i < N; i += G::THREADS) s_tw[i] = g_tw[N + i];
+    __syncthreads();
+  }
+  if (st14) {
     dft_regs<N1, N / N1>(v, s_tw);
 #pragma unroll
-    for (int k1 = 0; k1 < N1; ++k1) A[(N2 * k1 + q) * TY + yl] = k1 == 0 ? v[k1] : cmul(v[k1], s_tw[k1 * N2 + q]);
+    for (int k1 = 0; k1 < N1; ++k1)
+      A[(N2 * k1 + q) * TY + yl] = k1 == 0 ? v[k1] : cmul(v[k1], REG ? tw[k1] : s_tw[k1 * N2 + q]);
   }
   __syncthreads();
-  // forward, stage 2 (k1 = q): transform over j2; X[k1 + N1 k2] to row N2 k1 + k2, prescaled
-  {
-    V X[N2];
+  // forward, stage 2 (k1 = q): transform over j2; X[k1 + N1 k2] prescaled (!REG: to row N2 k1 + k2)
+  V X[N2];
 #pragma unroll
-    for (int j2 = 0; j2 < N2; ++j2) X[j2] = A[(N2 * q + j2) * TY + yl];
-    dft_regs<N2, N / N2>(X, s_tw);
-    hessian_prescale<float, N>(X, q, fy, fz, kp.inv_m_f);
-    constexpr int NYQ1 = (N / 2) % N1, NYQ2 = (N / 2) / N1;  // k_x = N/2 in slot NYQ2 of k1 = NYQ1
-    if (q == NYQ1) args.aux[HessAux<N>::kx_nyq + (int64_t)kz * N + ky] = cscale(X[NYQ2], (float)(N / 2));
+  for (int j2 = 0; j2 < N2; ++j2) X[j2] = A[(N2 * q + j2) * TY + yl];
+  dft_regs<N2, N / N2>(X, s_tw);
+  hessian_prescale<float, N>(X, q, fy, fz, kp.inv_m_f);
+  constexpr int NYQ1 = (N / 2) % N1, NYQ2 = (N / 2) / N1;  // k_x = N/2 in slot NYQ2 of k1 = NYQ1
+  if (q == NYQ1) args.aux[HessAux<N>::kx_nyq + (int64_t)kz * N + ky] = cscale(X[NYQ2], (float)(N / 2));
+  if constexpr (!REG) {
 #pragma unroll
     for (int k2 = 0; k2 < N2; ++k2) A[(N2 * q + k2) * TY + yl] = X[k2];
+    __syncthreads();
   }
-  __syncthreads();
   const float ikf = kp.local_only ? 0.f : 1.f / kp.kbkf_f;
   const bool need_abs = kz == N / 2 || (ky0 <= N / 2 && N / 2 < ky0 + TY);
 #pragma unroll 1
   for (int o = 0; o < (need_abs ? 4 : 3); ++o) {
+    // REG: the outputs alternate between the two tiles, one barrier each
+    V* T = REG && (o & 1) ? A : B;
     // inverse, stage 1 (k1 = q): multiplier as read, conj, transform over k2, twiddle
     {
-      V X[N2], Y[N2];
+      V Y[N2];
+      if constexpr (!REG) {
 #pragma unroll
-      for (int k2 = 0; k2 < N2; ++k2) X[k2] = A[(N2 * q + k2) * TY + yl];
+        for (int k2 = 0; k2 < N2; ++k2) X[k2] = A[(N2 * q + k2) * TY + yl];
+      }
       split_output<float, N>(X, o, q, nyz2, ikf, Y);
       conj_regs(Y);
       dft_regs<N2, N / N2>(Y, s_tw);
 #pragma unroll
-      for (int n2 = 0; n2 < N2; ++n2) B[(N2 * q + n2) * TY + yl] = n2 == 0 ? Y[n2] : cmul(Y[n2], s_tw[q * N2 + n2]);
+      for (int n2 = 0; n2 < N2; ++n2)
+        T[(N2 * q + n2) * TY + yl] = n2 == 0 ? Y[n2] : cmul(Y[n2], REG ? tw[n2] : s_tw[q * N2 + n2]);
     }
     __syncthreads();
     // inverse, stage 2 (n2 = q): transform over k1, conj, x = N2 n1 + n2 to global
     if (st14) {
       V w[N1];
 #pragma unroll
-      for (int k1 = 0; k1 < N1; ++k1) w[k1] = B[(N2 * k1 + q) * TY + yl];
+      for (int k1 = 0; k1 < N1; ++k1) w[k1] = T[(N2 * k1 + q) * TY + yl];
       dft_regs<N1, N / N1>(w, s_tw);
       if (o < 3) {
         V* plane = split_dst(args.out, o) + (int64_t)kz * N * N;
@@ -758,7 +776,7 @@ __global__ void __launch_bounds__(XSGeom<N>::THREADS, XSGeom<N>::MINB)
         for (int n1 = 0; n1 < N1; ++n1) split_store_abs<float, N>(args.aux, kz, ky, N2 * n1 + q, cconj(w[n1]));
       }
     }
-    __syncthreads();
+    if constexpr (!REG) __syncthreads();
   }
 }
 

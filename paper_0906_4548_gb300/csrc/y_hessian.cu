@@ -96,10 +96,10 @@ __global__ void __launch_bounds__(YHGeom<T, N>::THREADS, YHGeom<T, N>::MINB)
       // data convert the product once; the FP64 pipe is what bounds them)
       const float cA = o == 0 ? 1.f : 0.f;
       const float cB = o == 2 ? (nyq_z ? (float)(N / 2) : fz) : o == 3 ? 1.f : 0.f;
-      const float cC = o == 1 ? fz * fz : o == 4 ? (nyq_z ? (float)(N / 2) : fz) : 0.f;
+      const float cC = o == 1 ? fz * fz : o == 4 ? (nyq_z ? (float)(N / 2) : fz) : o == 5 ? 1.f : 0.f;
       const bool abs_y = nyq_z && o == 2;
       V v[N1];
-      if (o == 5) {
+      if (sizeof(T) == 8 && o == 5) {
 #pragma unroll
         for (int j1 = 0; j1 < N1; ++j1) v[j1] = cconj(g[j1]);
       } else {
