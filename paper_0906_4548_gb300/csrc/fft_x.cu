@@ -27,6 +27,7 @@
 #include <cooperative_groups.h>
 
 #include "adjoint_rc.cuh"
+#include "eft.cuh"
 #include "fft_core.cuh"
 #include "kernels.cuh"
 #include "reduce.cuh"
@@ -215,6 +216,44 @@ __device__ __forceinline__ void split_store_abs(vec2_t<T>* aux, int kz, int ky, 
   if (kz == N / 2) aux[HessAux<N>::kz_nyq + (int64_t)x * N + ky] = v;
 }
 
+// Sums of a P(k) shell: sqrt(n2) and |a|^2 (/ n2^2), as float pairs for FP32 data.
+template <typename T> struct ShellSum {
+  double s = 0.0;
+  __device__ __forceinline__ void add_root(int n2, bool twice) {
+    const double r = sqrt((double)n2);
+    s += twice ? 2.0 * r : r;
+  }
+  __device__ __forceinline__ void add_norm(double2 a) { s += a.x * a.x + a.y * a.y; }
+  __device__ __forceinline__ void add_norm_over(double2 a, int n2) {
+    s += (a.x * a.x + a.y * a.y) / ((double)n2 * (double)n2);
+  }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <> struct ShellSum<float> {
+  FP s{0.f, 0.f};
+  __device__ __forceinline__ void add_root(int n2, bool twice) {
+    // sqrt(n2) = r + (n2 - r^2) / (2 r), the remainder exact (n2 < 2^24)
+    const float f = (float)n2, r = sqrtf(f);
+    float lo = fmaf(-r, r, f) / (2.f * r), hi = r;
+    if (twice) {
+      hi *= 2.f;
+      lo *= 2.f;
+    }
+    fp_acc(s, FP{hi, lo});
+  }
+  __device__ __forceinline__ void add_norm(float2 a) {
+    FP p = fp_prod(a.x, a.x);
+    fp_acc(p, fp_prod(a.y, a.y));
+    fp_acc(s, p);
+  }
+  __device__ __forceinline__ void add_norm_over(float2 a, int n2) {
+    const double q = (double)a.x * a.x + (double)a.y * a.y, v = q / ((double)n2 * (double)n2);
+    const float hi = (float)v;
+    fp_acc(s, FP{hi, (float)(v - (double)hi)});
+  }
+  __device__ __forceinline__ double value() const { return (double)s.hi + (double)s.lo; }
+};
+
 template <typename T, int RB> struct XBatch {
   XArgs<T> a[RB];
 };
@@ -233,16 +272,12 @@ __global__ void __launch_bounds__(XGeom<T, N>::THREADS, XGeom<T, N>::MIN_BLOCKS)
   // shared memory so the output loop does not hold 2 * N2 extra registers
   T* s_inv = reinterpret_cast<T*>(s_T + N * TY);               // N2 * THREADS
   T* s_ikb = s_inv + N2 * XGeom<T, N>::THREADS;                // N2 * THREADS
-  // P(k) operations (which use neither table): per-warp shell sums
-  // [warp][NBS][nbins] and a per-warp staging row [warp][32][NBS]
-  constexpr int NW = XGeom<T, N>::THREADS / 32;
+  // P(k) operations (which use neither table): the transpose buffer has N more values (padded
+  // rows), then the shell sums of two halves of the columns, [2][NBS][nbins]
   constexpr int NBS = OP == XOP_PK_BRANE ? 4 : 3;  // sums per shell
-  double* s_bins = reinterpret_cast<double*>(s_inv);
+  double* s_bins = reinterpret_cast<double*>(s_T + N * (TY + 1));
   V* s_T2 = reinterpret_cast<V*>(s_inv);  // the Hessian op's second transpose buffer (N * TY)
-  double* s_stage = s_bins + NW * NBS * args.nbins;
   load_twiddles(s_tw, g_tw, N);
-  if (OP == XOP_PK || OP == XOP_PK_BRANE)
-    for (int i = threadIdx.x; i < NW * NBS * args.nbins; i += blockDim.x) s_bins[i] = 0.0;
   const int yl = threadIdx.x % TY;
   const int lane = threadIdx.x / TY;
   const int kz = blockIdx.y;
@@ -261,51 +296,78 @@ __global__ void __launch_bounds__(XGeom<T, N>::THREADS, XGeom<T, N>::MIN_BLOCKS)
   if (OP == XOP_PHI_FORCE && kp.gravity == 0) x_forward<T, N>(args.in1, kz, ky0, lane, yl, s_T, s_tw, X1);
 
   if (OP == XOP_PK || OP == XOP_PK_BRANE) {
-    // Shell sums in a fixed order, so that P(k) is the same bits on every run:
-    // per register slot, the lanes of a warp that fall in one shell are summed
-    // by the lowest of them in lane order into that warp's own shell row (the
-    // shells of different groups differ, so no two lanes write one address);
-    // the warps' rows are then added in warp order.
-    const double norm = kp.box * kp.box * kp.box * kp.inv_m * kp.inv_m;
-    const double w = (kz == 0 || kz == N / 2) ? 1.0 : 2.0;
-    const int wl = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    double* wbins = s_bins + wid * NBS * args.nbins;
-    double* stage = s_stage + wid * 32 * NBS;
-    __syncthreads();  // the bins are zeroed
+    // Shell sums in a fixed order, so that P(k) is the same bits on every run.  Shell b holds the modes
+    // with n^2 in [b^2 - b + 1, b^2 + b] (round(|n|) = b), on a column (ky, kz) one run of |kx|.  The
+    // CTA's spectrum goes to shared memory and one thread per shell and half of the columns walks
+    // its runs; the halves are then added.  FP32 data sum as float pairs (about 48 bits), as the
+    // other reductions do, since FP64 instructions are what a per-mode FP64 sum waits for.
+    constexpr int PP = TY + 1;  // padded row: threads of neighbouring shells read neighbouring kx
+    constexpr int HALVES = TY >= 2 ? 2 : 1, CPH = TY / HALVES;
+    int e = 0;  // FP32 data are scaled by 2^-e, so that their squares neither overflow nor underflow
+    if constexpr (sizeof(T) == 4) {
+      __shared__ float s_max[32];
+      float m = 0.f;
 #pragma unroll
-    for (int k2 = 0; k2 < N2; ++k2) {
-      const int nx = signed_index(lane + N1 * k2, N);
-      const int n2 = nx * nx + ny * ny + nz * nz;
-      const double nm = sqrt((double)n2);
-      int b = (int)floor(nm + 0.5);
-      if (n2 == 0 || b < 1 || b > args.nbins) b = 0;
-      const double p = ((double)X0[k2].x * X0[k2].x + (double)X0[k2].y * X0[k2].y) * norm;
-      stage[wl * NBS + 0] = w;
-      stage[wl * NBS + 1] = w * nm * (2.0 * M_PI / kp.box);
-      stage[wl * NBS + 2] = w * p;
-      if (OP == XOP_PK_BRANE) stage[wl * NBS + 3] = n2 ? w * p / ((double)n2 * (double)n2) : 0.0;
-      const unsigned group = __match_any_sync(0xffffffffu, b);
-      __syncwarp();
-      if (b != 0 && wl == __ffs(group) - 1) {
-        double acc[NBS];
+      for (int k2 = 0; k2 < N2; ++k2) m = fmaxf(m, fmaxf(fabsf(X0[k2].x), fabsf(X0[k2].y)));
 #pragma unroll
-        for (int c = 0; c < NBS; ++c) acc[c] = 0.0;
-        for (unsigned g = group; g; g &= g - 1) {
-          const int l = __ffs(g) - 1;
+      for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+      if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = m;
+      __syncthreads();
+      for (int i = 0; i < (int)(blockDim.x + 31) / 32; ++i) m = fmaxf(m, s_max[i]);
+      if (m > 0.f && isfinite(m)) e = max(ilogbf(m), -120);
+      const float sc = scalbnf(1.f, -e);
 #pragma unroll
-          for (int c = 0; c < NBS; ++c) acc[c] += stage[l * NBS + c];
+      for (int k2 = 0; k2 < N2; ++k2) X0[k2] = cscale(X0[k2], sc);
+    }
+#pragma unroll
+    for (int k2 = 0; k2 < N2; ++k2) s_T[(lane + N1 * k2) * PP + yl] = X0[k2];
+    __syncthreads();
+    for (int i = threadIdx.x; i < HALVES * args.nbins; i += blockDim.x) {
+      const int h = i / args.nbins, b = i % args.nbins + 1;
+      ShellSum<T> sk, sp, sb;
+      int cnt = 0;
+      for (int cc = 0; cc < CPH; ++cc) {
+        const int col = h * CPH + cc;
+        const int nyc = signed_index(ky0 + col, N);
+        const int r2 = nyc * nyc + nz * nz;
+        const int hi = b * b + b - r2;
+        if (hi < 0) continue;
+        int lo = b * b - b + 1 - r2;
+        if (lo < 0) lo = 0;
+        int k0 = (int)sqrtf((float)lo);  // the run |kx| = k0 .. k1 with kx^2 in [lo, hi]
+        while (k0 * k0 < lo) ++k0;
+        while (k0 > 0 && (k0 - 1) * (k0 - 1) >= lo) --k0;
+        for (int kx = k0; kx <= N / 2 && kx * kx <= hi; ++kx) {
+          const int n2 = r2 + kx * kx;
+          const V a = s_T[kx * PP + col];
+          const bool two = kx != 0 && kx != N / 2;
+          sk.add_root(n2, two);
+          sp.add_norm(a);
+          if (OP == XOP_PK_BRANE) sb.add_norm_over(a, n2);
+          ++cnt;
+          if (two) {
+            const V m = s_T[(N - kx) * PP + col];
+            sp.add_norm(m);
+            if (OP == XOP_PK_BRANE) sb.add_norm_over(m, n2);
+            ++cnt;
+          }
         }
-#pragma unroll
-        for (int c = 0; c < NBS; ++c) wbins[c * args.nbins + b - 1] += acc[c];
       }
-      __syncwarp();
+      double* o = s_bins + h * NBS * args.nbins + b - 1;
+      o[0] = (double)cnt;
+      o[args.nbins] = sk.value();
+      o[2 * args.nbins] = sp.value();
+      if (OP == XOP_PK_BRANE) o[3 * args.nbins] = sb.value();
     }
     __syncthreads();
+    const double norm = scalbn(kp.box * kp.box * kp.box * kp.inv_m * kp.inv_m, 2 * e);
+    const double w = (kz == 0 || kz == N / 2) ? 1.0 : 2.0;
     const int64_t blk = (int64_t)blockIdx.y * gridDim.x + blockIdx.x;
     for (int i = threadIdx.x; i < NBS * args.nbins; i += blockDim.x) {
-      double t = 0.0;
-      for (int v = 0; v < NW; ++v) t += s_bins[v * NBS * args.nbins + i];
-      args.pk_partials[blk * NBS * args.nbins + i] = t;
+      double t = s_bins[i];
+      if (HALVES == 2) t += s_bins[NBS * args.nbins + i];
+      const int c = i / args.nbins;
+      args.pk_partials[blk * NBS * args.nbins + i] = c == 0 ? w * t : c == 1 ? w * (2.0 * M_PI / kp.box) * t : w * norm * t;
     }
     return;
   }
@@ -794,15 +856,14 @@ template <typename T, int N> int x_pass_blocks() { return (N / XGeom<T, N>::TY) 
 template <typename T, int N, int OP, int RB = 1>
 static void launch_x(const XArgs<T>* a, int count, const vec2_t<T>* tw, cudaStream_t s) {
   using G = XGeom<T, N>;
-  // the P(k) operations put their per-warp shell sums where the others keep
-  // their per-thread multiplier tables
+  // the P(k) operations put their shell sums where the others keep their per-thread multiplier tables
   constexpr bool PK = OP == XOP_PK || OP == XOP_PK_BRANE;
-  constexpr int NBS = OP == XOP_PK_BRANE ? 4 : 3, NW = G::THREADS / 32;
+  constexpr int NBS = OP == XOP_PK_BRANE ? 4 : 3;
   const size_t base = sizeof(vec2_t<T>) * (kTwiddleTables * N + (size_t)N * G::TY);
-  const size_t tables = PK ? sizeof(double) * NW * 32 * NBS
+  const size_t tables = PK ? sizeof(vec2_t<T>) * N
                             : ((OP == XOP_HESSIAN || OP == XOP_PHI_FORCE) ? sizeof(vec2_t<T>) * (size_t)N * G::TY
                                                                           : sizeof(T) * 2 * Split<N>::N2 * G::THREADS);
-  const size_t per_bin = PK ? sizeof(double) * NW * NBS : 0;
+  const size_t per_bin = PK ? sizeof(double) * 2 * NBS : 0;
   const size_t smem = base + tables + per_bin * a[0].nbins;
   if constexpr (OP == XOP_HESSIAN && sizeof(T) == 4 && N <= 256) {
     launch_xs<N, RB>(a, count, tw, s);  // the shared-memory version of the same pass

@@ -42,18 +42,17 @@ __global__ void __launch_bounds__(256) k_finalize(const double* __restrict__ par
       for (int c = 0; c < 4; ++c) out[c] = v[c];
     return;
   }
-  for (int c = 0; c < ncomp; ++c) {
-    double v[1] = {0.0};
-    for (int b = threadIdx.x; b < nblocks; b += blockDim.x) v[0] += partials[(int64_t)b * ncomp + c];
-    block_sum<1>(v);
-    if (threadIdx.x == 0) out[c] = v[0];
-    __syncthreads();
-  }
+  // one block per component: the hundreds of sums of P(k) took 380 us in one block (256^3, 128 shells)
+  const int c = blockIdx.x;
+  double v[1] = {0.0};
+  for (int b = threadIdx.x; b < nblocks; b += blockDim.x) v[0] += partials[(int64_t)b * ncomp + c];
+  block_sum<1>(v);
+  if (threadIdx.x == 0) out[c] = v[0];
 }
 
 void launch_finalize(const double* partials, int nblocks, int ncomp, double* out, cudaStream_t s,
                      const int* skip) {
-  k_finalize<<<1, 256, 0, s>>>(partials, nblocks, ncomp, out, skip);
+  k_finalize<<<ncomp == 4 ? 1 : ncomp, 256, 0, s>>>(partials, nblocks, ncomp, out, skip);
 }
 
 // Batched one-component sums: realisation r = blockIdx.y (k_sum) or blockIdx.x (finalize).
