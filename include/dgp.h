@@ -429,7 +429,8 @@ int dgp_brane_spectra(dgp_ctx *c, int nbins, double *k, double *pc, double *pC, 
  *               cell_start[n^3] = parts->n); synchronised on return when given.
  * The first call, and any call with more particles than before, allocates
  * 4 + 6 sizeof(real) bytes per particle and 12 n^3 bytes of workspace; the
- * sort itself goes through those copies (the six arrays are copied back).
+ * sort goes through records of a particle's values in it, which are then split
+ * into the six arrays.
  * DGP_E_INVALID for a bad argument, DGP_E_NOMEM, DGP_E_CUDA. */
 int dgp_sort_particles(dgp_ctx *c, dgp_particles *parts, int32_t *cell_start);
 

@@ -381,9 +381,9 @@ class Engine : public EngineBase {
   int64_t hp_n = 0;
   // cell sort: key and permuted copies per particle, counts / starts / cursors per cell
   int* srt_key = nullptr;
-  T* srt_tmp[6] = {};
+  T* srt_tmp[2] = {};           // records of 4 and of 2 values per particle
   int64_t srt_np = 0;
-  int* srt_cell = nullptr;      // [3][M]: count, start, cursor
+  int* srt_cell = nullptr;      // [3][M]: count, cursor; the third is not used
   int* srt_sums = nullptr;
   int64_t nsteps = 0;           // pm_step calls since init / reset
   // adjoint workspace (allocated on the first dgp_solve_adjoint)
@@ -423,7 +423,7 @@ class Engine : public EngineBase {
       if (pair_exec[i]) cudaGraphExecDestroy(pair_exec[i]);
     if (class_exec) cudaGraphExecDestroy(class_exec);
     set_blocking(false);
-    for (int i = 0; i < 6; ++i) cudaFree(srt_tmp[i]);
+    for (int i = 0; i < 2; ++i) cudaFree(srt_tmp[i]);
     cudaFreeHost(h_stats);
   }
 
@@ -907,24 +907,21 @@ class Engine : public EngineBase {
       DGP_CUDA(wait_stream());
       cudaFree(srt_key);
       srt_key = nullptr;
-      for (int i = 0; i < 6; ++i) { cudaFree(srt_tmp[i]); srt_tmp[i] = nullptr; }
+      for (int i = 0; i < 2; ++i) { cudaFree(srt_tmp[i]); srt_tmp[i] = nullptr; }
       srt_np = 0;
       if (cudaMalloc(&srt_key, sizeof(int) * np) != cudaSuccess) return DGP_E_NOMEM;
-      for (int i = 0; i < 6; ++i)
-        if (cudaMalloc(&srt_tmp[i], sizeof(T) * np) != cudaSuccess) return DGP_E_NOMEM;
+      for (int i = 0; i < 2; ++i)
+        if (cudaMalloc(&srt_tmp[i], sizeof(T) * (i == 0 ? 4 : 2) * np) != cudaSuccess) return DGP_E_NOMEM;
       srt_np = np;
     }
     ParticleSet<T> in{{(T*)pp->x, (T*)pp->y, (T*)pp->z, (T*)pp->px, (T*)pp->py, (T*)pp->pz}};
-    ParticleSet<T> out{{srt_tmp[0], srt_tmp[1], srt_tmp[2], srt_tmp[3], srt_tmp[4], srt_tmp[5]}};
-    const SortWork w{srt_key, srt_cell, srt_cell + M, srt_cell + 2 * M, srt_sums};
-    const double pb = sizeof(T) * 15.0 + 8.0;  // read x (3), key out/in, read 6, write 6
-    prof.run(KK_SORT, pb * np + 16.0 * M, stream, [&] { launch_cell_sort<T>(in, np, cic(), w, out, stream); });
+    const SortWork w{srt_key, srt_cell, srt_cell + M, srt_sums};
+    const double pb = sizeof(T) * 27.0 + 8.0;  // read x (3), key out/in, read 6, write 6, the records split
+    prof.run(KK_SORT, pb * np + (cell_start ? 16.0 : 12.0) * M, stream,
+             [&] { launch_cell_sort<T>(in, np, cic(), w, cell_start, srt_tmp[0], srt_tmp[1], stream); });
     DGP_CHECK_LAUNCH();
-    for (int i = 0; i < 6 && np > 0; ++i)
-      DGP_CUDA(cudaMemcpyAsync(in.p[i], out.p[i], sizeof(T) * np, cudaMemcpyDeviceToDevice, stream));
     if (cell_start) {
       const int total = (int)np;
-      DGP_CUDA(cudaMemcpyAsync(cell_start, w.start, sizeof(int) * M, cudaMemcpyDeviceToDevice, stream));
       DGP_CUDA(cudaMemcpyAsync(cell_start + M, &total, sizeof(int), cudaMemcpyHostToDevice, stream));
       DGP_CUDA(wait_stream());
     }

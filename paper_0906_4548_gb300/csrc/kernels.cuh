@@ -369,15 +369,15 @@ struct ParticleSet {
 struct SortWork {
   int* key;     // [np] cell of each particle
   int* count;   // [N^3] particles per cell
-  int* start;   // [N^3] exclusive scan of count: first slot of each cell
-  int* cursor;  // [N^3] scatter cursors
+  int* cursor;  // [N^3] scatter cursors (the exclusive scan of count)
   int* sums;    // [sort_scan_blocks(N^3)] chunk sums of the scan
 };
 int sort_scan_blocks(int64_t m);
-// Writes the particles of parts, ordered by cell, into tmp (no copy back).
+// Orders the particles by cell in place, through rec4 and rec2 (4 np and 2 np values, 16-byte
+// aligned); cell_start (may be null): the first N^3 entries, the first slot of each cell.
 template <typename T>
-void launch_cell_sort(const ParticleSet<T>& parts, int64_t np, CicParams cp, const SortWork& w,
-                      const ParticleSet<T>& tmp, cudaStream_t s);
+void launch_cell_sort(const ParticleSet<T>& parts, int64_t np, CicParams cp, const SortWork& w, int* cell_start,
+                      T* rec4, T* rec2, cudaStream_t s);
 // CIC deposit with warp-aggregated atomics over lanes that share a cell.
 template <typename T>
 void launch_cic_deposit_warp(const T* x, const T* y, const T* z, int64_t np, T* rho, CicParams cp,

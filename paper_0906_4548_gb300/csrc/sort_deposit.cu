@@ -4,7 +4,11 @@
 // the lower CIC corner, (i0x N + i0y) N + i0z, computed by the same cic_axis as
 // the deposit and the gather.  A histogram of keys, an exclusive scan of the
 // histogram and a scatter through atomic cursors give the particles ordered by
-// key; the order inside one cell is whatever the cursors hand out.
+// key; the order inside one cell is whatever the cursors hand out.  The scatter
+// writes a particle as two records (x, y, z, px and py, pz) instead of six
+// values: on particles in random order it is bound by the number of scattered
+// stores (27e9 a second measured), and a streaming pass then splits the records
+// into the caller's arrays, which a copy back would have to write anyway.
 //
 // Deposit (Eq. CIC) with warp-aggregated atomics: after a sort the particles
 // of one cell sit in adjacent lanes, and a warp issues one set of eight
@@ -79,18 +83,25 @@ __global__ void __launch_bounds__(1024) k_scan_top(int* __restrict__ sums, int n
   }
 }
 
+// cursor (and start, when wanted): the exclusive scan
 __global__ void __launch_bounds__(256) k_scan_chunks(const int* __restrict__ in, int64_t m,
                                                      const int* __restrict__ sums, int* __restrict__ start,
                                                      int* __restrict__ cursor) {
   __shared__ int s_w[8];
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const int64_t base = (int64_t)blockIdx.x * kScanChunk + threadIdx.x * 8;
-  int v[8], t = 0;
+  __align__(16) int v[8];
+  int t = 0;
+  // meshes have a multiple of 8 points, so a thread's 8 counts are all there or none
+  if (base < m) {
+    *reinterpret_cast<int4*>(v) = *reinterpret_cast<const int4*>(in + base);
+    *reinterpret_cast<int4*>(v + 4) = *reinterpret_cast<const int4*>(in + base + 4);
+  } else {
 #pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    v[j] = base + j < m ? in[base + j] : 0;
-    t += v[j];
+    for (int j = 0; j < 8; ++j) v[j] = 0;
   }
+#pragma unroll
+  for (int j = 0; j < 8; ++j) t += v[j];
   const int x = warp_inclusive_scan(t, lane);
   if (lane == 31) s_w[wid] = x;
   __syncthreads();
@@ -98,30 +109,63 @@ __global__ void __launch_bounds__(256) k_scan_chunks(const int* __restrict__ in,
   for (int w = 0; w < wid; ++w) run += s_w[w];
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
-    if (base + j < m) {
-      start[base + j] = run;
-      cursor[base + j] = run;
+    const int c = v[j];
+    v[j] = run;
+    run += c;
+  }
+  if (base < m) {
+    *reinterpret_cast<int4*>(cursor + base) = *reinterpret_cast<const int4*>(v);
+    *reinterpret_cast<int4*>(cursor + base + 4) = *reinterpret_cast<const int4*>(v + 4);
+    if (start && (reinterpret_cast<uintptr_t>(start) & 15) == 0) {
+      *reinterpret_cast<int4*>(start + base) = *reinterpret_cast<const int4*>(v);
+      *reinterpret_cast<int4*>(start + base + 4) = *reinterpret_cast<const int4*>(v + 4);
+    } else if (start) {  // the caller's array need only be aligned as int32
+#pragma unroll
+      for (int j = 0; j < 8; ++j) start[base + j] = v[j];
     }
-    run += v[j];
   }
 }
+
+template <typename T> struct Rec4 { T x, y, z, px; };
+template <typename T> struct Rec2 { T py, pz; };
+template <> struct __align__(16) Rec4<float> { float x, y, z, px; };
+template <> struct __align__(8) Rec2<float> { float py, pz; };
+template <> struct __align__(16) Rec4<double> { double x, y, z, px; };
+template <> struct __align__(16) Rec2<double> { double py, pz; };
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_scatter(const __grid_constant__ ParticleSet<T> in, int64_t np,
                                                  const int* __restrict__ key, int* __restrict__ cursor,
-                                                 const __grid_constant__ ParticleSet<T> out) {
+                                                 Rec4<T>* __restrict__ r4, Rec2<T>* __restrict__ r2) {
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < np; p += (int64_t)gridDim.x * blockDim.x) {
+    const Rec4<T> a{in.p[0][p], in.p[1][p], in.p[2][p], in.p[3][p]};
+    const Rec2<T> b{in.p[4][p], in.p[5][p]};
     const int dst = atomicAdd(cursor + key[p], 1);
-#pragma unroll
-    for (int c = 0; c < 6; ++c) out.p[c][dst] = in.p[c][p];
+    r4[dst] = a;
+    r2[dst] = b;
+  }
+}
+
+template <typename T>
+__global__ void __launch_bounds__(256) k_split_records(const Rec4<T>* __restrict__ r4, const Rec2<T>* __restrict__ r2,
+                                                       int64_t np, const __grid_constant__ ParticleSet<T> out) {
+  for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < np; p += (int64_t)gridDim.x * blockDim.x) {
+    const Rec4<T> a = r4[p];
+    const Rec2<T> b = r2[p];
+    out.p[0][p] = a.x;
+    out.p[1][p] = a.y;
+    out.p[2][p] = a.z;
+    out.p[3][p] = a.px;
+    out.p[4][p] = b.py;
+    out.p[5][p] = b.pz;
   }
 }
 
 int sort_scan_blocks(int64_t m) { return (int)((m + kScanChunk - 1) / kScanChunk); }
 
 template <typename T>
-void launch_cell_sort(const ParticleSet<T>& parts, int64_t np, CicParams cp, const SortWork& w,
-                      const ParticleSet<T>& tmp, cudaStream_t s) {
+void launch_cell_sort(const ParticleSet<T>& parts, int64_t np, CicParams cp, const SortWork& w, int* cell_start,
+                      T* rec4, T* rec2, cudaStream_t s) {
   const int64_t m = (int64_t)cp.n * cp.n * cp.n;
   cudaMemsetAsync(w.count, 0, sizeof(int) * m, s);
   int64_t blocks = (np + 255) / 256;
@@ -132,8 +176,13 @@ void launch_cell_sort(const ParticleSet<T>& parts, int64_t np, CicParams cp, con
   const int nb = sort_scan_blocks(m);
   k_scan_sums<<<nb, 256, 0, s>>>(w.count, m, w.sums);
   k_scan_top<<<1, 1024, 0, s>>>(w.sums, nb);
-  k_scan_chunks<<<nb, 256, 0, s>>>(w.count, m, w.sums, w.start, w.cursor);
-  if (np > 0) k_scatter<T><<<(unsigned)blocks, 256, 0, s>>>(parts, np, w.key, w.cursor, tmp);
+  k_scan_chunks<<<nb, 256, 0, s>>>(w.count, m, w.sums, cell_start, w.cursor);
+  if (np > 0) {
+    Rec4<T>* r4 = reinterpret_cast<Rec4<T>*>(rec4);
+    Rec2<T>* r2 = reinterpret_cast<Rec2<T>*>(rec2);
+    k_scatter<T><<<(unsigned)blocks, 256, 0, s>>>(parts, np, w.key, w.cursor, r4, r2);
+    k_split_records<T><<<(unsigned)blocks, 256, 0, s>>>(r4, r2, np, parts);
+  }
 }
 
 // ---------------------------------------------------------------- deposit
@@ -250,8 +299,8 @@ void launch_cic_deposit_batch(const DepositArgs<T>* a, int count, cudaStream_t s
 }
 
 #define DGP_INST_SORT(T)                                                                                   \
-  template void launch_cell_sort<T>(const ParticleSet<T>&, int64_t, CicParams, const SortWork&,             \
-                                    const ParticleSet<T>&, cudaStream_t);                                  \
+  template void launch_cell_sort<T>(const ParticleSet<T>&, int64_t, CicParams, const SortWork&, int*, T*,   \
+                                    T*, cudaStream_t);                                                      \
   template void launch_cic_deposit_warp<T>(const T*, const T*, const T*, int64_t, T*, CicParams, cudaStream_t); \
   template void launch_cic_deposit_batch<T>(const DepositArgs<T>*, int, cudaStream_t);
 DGP_INST_SORT(float)
