@@ -1992,40 +1992,58 @@ class Engine : public EngineBase {
     if ((rc = forward_zy((const T*)delta, s6[5], ZPrologue{nullptr, 0.0, 0}))) return rc;
     const Coef c = coefficients(1.0, cosmo.omega_m0, p.rc_H0);
     const KParams kp = kparams(c, p.gravity);
+    // modes with lo < |n| < hi as whole-number bounds on |n|^2 (the smallest n2 whose root passes each)
+    auto bound = [](double r, bool strict) {
+      if (!(r > 0.0)) return strict && r == 0.0 ? 1 : 0;
+      const double lim = 3.0 * (N / 2) * (N / 2) + 1.0;
+      if (!(r * r < lim)) return (int)lim;
+      int n = std::max(0, (int)(r * r) - 2);
+      while (strict ? !(sqrt((double)n) > r) : sqrt((double)n) < r) ++n;
+      return n;
+    };
     auto shell = [&](double kc, T* d, T* ind) -> int {
       prof.run(KK_X_OTHER, 3 * SB, stream, [&] {
-        launch_fft_x_op<T, N>(XOP_SHELL, s6[5], nullptr, fs(s6, 2), 0, kp, nullptr, 0, (kc - 0.5 * dk) / kf,
-                              (kc + 0.5 * dk) / kf, tw, stream);
+        launch_fft_x_op<T, N>(XOP_SHELL, s6[5], nullptr, fs(s6, 2), 0, kp, nullptr, 0, bound((kc - 0.5 * dk) / kf, true),
+                              bound((kc + 0.5 * dk) / kf, false), tw, stream);
       });
       T* outs[2] = {d, ind};
       return inverse_yz(s6, outs, 2);
     };
-    auto dot3 = [&](const T* x, const T* y, const T* z, double* hv) -> int {
-      prof.run(KK_REDUCE, (z ? 3 : 2) * RB, stream,
-               [&] { launch_product3_sum<T>(x, y, z, M, partials, nblocks, stream); });
-      prof.run(KK_REDUCE, 8.0 * nblocks, stream, [&] { launch_finalize(partials, nblocks, 1, d_misc + 2, stream); });
+    // the sums of a pass into slot i of d_pk (four doubles a slot)
+    auto sums = [&](bool triple, int i) -> int {
+      T* const f[6] = {rH[0], rH[1], rH[2], rH[3], triple ? rH[4] : nullptr, triple ? rH[5] : nullptr};
+      prof.run(KK_REDUCE, (triple ? 6 : 4) * RB, stream,
+               [&] { launch_bispec_sums<T>(f, d_misc + 2, M, partials, nblocks, stream); });
+      prof.run(KK_REDUCE, 32.0 * nblocks, stream, [&] { launch_finalize(partials, nblocks, 4, d_pk + 4 * i, stream); });
       DGP_CHECK_LAUNCH();
-      int r2 = fetch(d_misc + 2, 1);
-      *hv = h_stats[0];
-      return r2;
+      return DGP_OK;
     };
-    if ((rc = shell(k1, rH[0], rH[1]))) return rc;
-    if ((rc = shell(k2, rH[2], rH[3]))) return rc;
-    double d11, i11, d22, i22;
-    if ((rc = dot3(rH[0], rH[0], nullptr, &d11)) || (rc = dot3(rH[1], rH[1], nullptr, &i11))) return rc;
-    if ((rc = dot3(rH[2], rH[2], nullptr, &d22)) || (rc = dot3(rH[3], rH[3], nullptr, &i22))) return rc;
+    if ((rc = reduce_sum((const T*)delta, true, d_misc + 2))) return rc;
+    if ((rc = shell(k1, rH[0], rH[1])) || (rc = shell(k2, rH[2], rH[3])) || (rc = sums(false, 0))) return rc;
     const double L3M2 = p.box * p.box * p.box / ((double)M * (double)M);
-    const double P1 = L3M2 * d11 / i11, P2 = L3M2 * d22 / i22;
-    for (int i = 0; i < ntheta; ++i) {
-      const double k3 = sqrt(k1 * k1 + k2 * k2 + 2.0 * k1 * k2 * cos(theta[i]));
-      if ((rc = shell(k3, rH[4], rH[5]))) return rc;
-      double ddd, iii, d33, i33;
-      if ((rc = dot3(rH[0], rH[2], rH[4], &ddd)) || (rc = dot3(rH[1], rH[3], rH[5], &iii))) return rc;
-      if ((rc = dot3(rH[4], rH[4], nullptr, &d33)) || (rc = dot3(rH[5], rH[5], nullptr, &i33))) return rc;
-      const double P3 = L3M2 * d33 / i33;
-      const double L6M3 = pow(p.box, 6) / ((double)M * (double)M * (double)M);
-      b[i] = L6M3 * ddd / iii;
-      q[i] = b[i] / (P1 * P2 + P2 * P3 + P3 * P1);
+    const double L6M3 = pow(p.box, 6) / ((double)M * (double)M * (double)M);
+    // angles in groups whose sums fit d_pk (N / 2 slots), read once per group
+    double h[4 * (N / 2)], P1 = 0.0, P2 = 0.0;
+    int first = 1;  // slot 0 holds the sums of k1 and k2 in the first group
+    for (int i0 = 0; i0 < ntheta || first; first = 0) {
+      const int cnt = std::min(ntheta - i0, N / 2 - first);
+      for (int i = 0; i < cnt; ++i) {
+        const double k3 = sqrt(k1 * k1 + k2 * k2 + 2.0 * k1 * k2 * cos(theta[i0 + i]));
+        if ((rc = shell(k3, rH[4], rH[5])) || (rc = sums(true, first + i))) return rc;
+      }
+      DGP_CUDA(cudaMemcpyAsync(h, d_pk, sizeof(double) * 4 * (first + cnt), cudaMemcpyDeviceToHost, stream));
+      DGP_CUDA(wait_stream());
+      if (first) {
+        P1 = L3M2 * h[0] / h[1];
+        P2 = L3M2 * h[2] / h[3];
+      }
+      for (int i = 0; i < cnt; ++i) {
+        const double* t = h + 4 * (first + i);
+        const double P3 = L3M2 * t[2] / t[3];
+        b[i0 + i] = L6M3 * t[0] / t[1];
+        q[i0 + i] = b[i0 + i] / (P1 * P2 + P2 * P3 + P3 * P1);
+      }
+      i0 += cnt;
     }
     return DGP_OK;
   }

@@ -52,7 +52,7 @@ template <typename T> struct XArgs {
   KParams kp;
   double* pk_partials;
   int nbins;
-  double shell_lo, shell_hi;
+  int shell_lo, shell_hi;  // XOP_SHELL: the modes with shell_lo <= n^2 < shell_hi
   const int* skip;
   vec2_t<T>* aux;  // XOP_HESSIAN: the Nyquist coefficients (HessAux)
   FieldSet<T> in;  // adjoint ops: input spectra
@@ -289,6 +289,14 @@ __global__ void __launch_bounds__(XGeom<T, N>::THREADS, XGeom<T, N>::MIN_BLOCKS)
   const KParams& kp = args.kp;
   const T kf = kc<T>(2.0 * M_PI / kp.box, kp.kf_f);
   __syncthreads();
+  if (OP == XOP_SHELL && nz * nz >= args.shell_hi) {  // no mode of the plane is in the shell
+    for (int i = threadIdx.x; i < N * TY; i += blockDim.x) {
+      const int64_t at = ((int64_t)kz * N + i / TY) * N + ky0 + i % TY;
+      args.out.p[0][at] = cmake<V>((T)0, (T)0);
+      args.out.p[1][at] = cmake<V>((T)0, (T)0);
+    }
+    return;
+  }
 
   V X0[N2], X1[N2];
   constexpr bool ADJ = OP == XOP_ADJ_PHI || OP == XOP_ADJ_COMBINE || OP == XOP_ZEL_ADJ || OP == XOP_RC;
@@ -689,8 +697,7 @@ __global__ void __launch_bounds__(XGeom<T, N>::THREADS, XGeom<T, N>::MIN_BLOCKS)
           r = cscale(X0[k2], sfac);
           if (o == 1) r = cscale(r, (T)1 / (kc<T>(kp.alpha, kp.alpha_f) - kc<T>(kp.c2, kp.c2_f) * ikb));
         } else if (OP == XOP_SHELL) {
-          const double nm = sqrt((double)n2);
-          if (nm > args.shell_lo && nm < args.shell_hi)
+          if (n2 >= args.shell_lo && n2 < args.shell_hi)
             r = (o == 0) ? cscale(X0[k2], inv_m) : cmake<V>(inv_m, (T)0);
         } else {  // XOP_PHI_FORCE
           const T kmag = kf * sqrt((T)n2);
@@ -902,7 +909,7 @@ void launch_fft_x_batch(int op, const XReal<T>* rz, int count, const vec2_t<T>* 
 
 template <typename T, int N>
 void launch_fft_x_op(int op, const vec2_t<T>* in0, const vec2_t<T>* in1, const FieldSet<T>& out, int nout_mask,
-                     const KParams& kp, double* pk_partials, int nbins, double shell_lo, double shell_hi,
+                     const KParams& kp, double* pk_partials, int nbins, int shell_lo, int shell_hi,
                      const vec2_t<T>* tw, cudaStream_t s, const int* skip, vec2_t<T>* aux) {
   XArgs<T> a{};
   a.skip = skip;

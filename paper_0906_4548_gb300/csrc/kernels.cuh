@@ -109,12 +109,12 @@ void launch_fft_z_c2r_batch(const FieldSet<T>* in, const FieldSet<T>* out, int n
 // partials (pk_partials, 3 * nbins doubles per block: modes, sum |k|,
 // sum |X|^2 box^3 / N^6); XOP_PK_BRANE adds sum |X|^2 box^3 / N^6 / |n|^4
 // (4 * nbins per block).  For XOP_SHELL the
-// op is a shell indicator on |k| (shell_lo <= |k|/k_f < shell_hi) applied to
+// op is the shell indicator shell_lo <= |n|^2 < shell_hi (n = k / k_f) applied to
 // input 0 (out 0) and the indicator itself (out 1).
 template <typename T, int N>
 void launch_fft_x_op(int op, const vec2_t<T>* in0, const vec2_t<T>* in1, const FieldSet<T>& out,
-                     int nout_mask, const KParams& kp, double* pk_partials, int nbins, double shell_lo,
-                     double shell_hi, const vec2_t<T>* tw, cudaStream_t s, const int* skip = nullptr,
+                     int nout_mask, const KParams& kp, double* pk_partials, int nbins, int shell_lo,
+                     int shell_hi, const vec2_t<T>* tw, cudaStream_t s, const int* skip = nullptr,
                      vec2_t<T>* aux = nullptr);
 
 // Adjoint x-passes (several y-transformed input spectra):
@@ -317,9 +317,13 @@ void launch_fill(T* a, int64_t m, T v, cudaStream_t s);
 template <typename T>
 void launch_sub_mean(const T* in, T* out, int64_t m, const double* sum, cudaStream_t s);
 
+// Sums of the bispectrum estimator in one pass, partials[block][4] (nblocks blocks):
+//  f[4], f[5] null: sum f0^2, f1^2, f2^2, f3^2;
+//  else, with fields (d1, i1, d2, i2, d3, i3): sum d1 d2 d3, i1 i2 i3, d3^2, i3^2.
+// abs_sum / m, the mean |.| of the measured field, sets the power of two by which FP32 fields d are
+// scaled before they are multiplied (undone in the sums).
 template <typename T>
-void launch_product3_sum(const T* a, const T* b, const T* c, int64_t m, double* partials,
-                         int nblocks, cudaStream_t s);
+void launch_bispec_sums(T* const* f6, const double* abs_sum, int64_t m, double* partials, int nblocks, cudaStream_t s);
 
 // Particles.
 struct CicParams {

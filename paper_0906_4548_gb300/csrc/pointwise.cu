@@ -8,6 +8,7 @@
 #include "common.cuh"
 #include "kernels.cuh"
 #include "cic.cuh"
+#include "eft.cuh"
 #include "reduce.cuh"
 #include "relax_control.cuh"
 
@@ -249,24 +250,73 @@ void launch_sum(const T* a, int64_t m, bool absval, double* partials, int nblock
   k_sum<T><<<nblocks, 256, 0, s>>>(a, m, absval ? 1 : 0, partials);
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256) k_product3(const T* __restrict__ a, const T* __restrict__ b,
-                                                  const T* __restrict__ c, int64_t m, double* __restrict__ partials) {
-  double acc = 0.0;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-    double v = (double)a[i] * (double)b[i];
-    if (c) v *= (double)c[i];
-    acc += v;
+// Running sum of products: FP32 factors multiply and add as float pairs (about 48 bits; FP64
+// instructions on the converted factors took 14 us a product sum at 128^3, four sums an angle),
+// FP64 factors in FP64.
+template <typename T> struct ProductSum {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double a, double b) { s += a * b; }
+  __device__ __forceinline__ void add(double a, double b, double c) { s += a * b * c; }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <> struct ProductSum<float> {
+  FP s{0.f, 0.f};
+  __device__ __forceinline__ void add(float a, float b) { fp_acc(s, fp_prod(a, b)); }
+  __device__ __forceinline__ void add(float a, float b, float c) {
+    const FP p = fp_prod(a, b);
+    FP q = fp_prod(p.hi, c);
+    q.lo = fmaf(p.lo, c, q.lo);
+    fp_acc(s, q);
   }
-  double v[1] = {acc};
-  block_sum<1>(v);
-  if (threadIdx.x == 0) partials[blockIdx.x] = v[0];
+  __device__ __forceinline__ double value() const { return (double)s.hi + (double)s.lo; }
+};
+
+template <typename T> struct BispecFields {
+  const T* f[6];
+};
+template <typename T, bool TRIPLE>
+__global__ void __launch_bounds__(256) k_bispec_sums(const __grid_constant__ BispecFields<T> a,
+                                                     const double* __restrict__ abs_sum, int64_t m,
+                                                     double* __restrict__ partials) {
+  // the fields d are filtered parts of the measured field: scaled by its size, their products
+  // neither overflow nor underflow
+  int e = 0;
+  if constexpr (sizeof(T) == 4) {
+    const double mean = abs_sum[0] / (double)m;
+    if (mean > 0.0 && isfinite(mean)) e = min(max(ilogb(mean), -120), 120);
+  }
+  const T sc = (T)scalbn(1.0, -e);
+  ProductSum<T> s0, s1, s2, s3;
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
+    const T d1 = a.f[0][i] * sc, i1 = a.f[1][i], d2 = a.f[2][i] * sc, i2 = a.f[3][i];
+    if constexpr (TRIPLE) {
+      const T d3 = a.f[4][i] * sc, i3 = a.f[5][i];
+      s0.add(d1, d2, d3);
+      s1.add(i1, i2, i3);
+      s2.add(d3, d3);
+      s3.add(i3, i3);
+    } else {
+      s0.add(d1, d1);
+      s1.add(i1, i1);
+      s2.add(d2, d2);
+      s3.add(i2, i2);
+    }
+  }
+  double v[4] = {s0.value(), s1.value(), s2.value(), s3.value()};
+  v[0] = scalbn(v[0], TRIPLE ? 3 * e : 2 * e);
+  v[2] = scalbn(v[2], 2 * e);
+  block_sum<4>(v);
+  if (threadIdx.x == 0)
+    for (int k = 0; k < 4; ++k) partials[4 * (int64_t)blockIdx.x + k] = v[k];
 }
 
 template <typename T>
-void launch_product3_sum(const T* a, const T* b, const T* c, int64_t m, double* partials, int nblocks,
-                         cudaStream_t s) {
-  k_product3<T><<<nblocks, 256, 0, s>>>(a, b, c, m, partials);
+void launch_bispec_sums(T* const* f6, const double* abs_sum, int64_t m, double* partials, int nblocks,
+                        cudaStream_t s) {
+  BispecFields<T> a;
+  for (int i = 0; i < 6; ++i) a.f[i] = f6[i];
+  if (f6[4]) k_bispec_sums<T, true><<<nblocks, 256, 0, s>>>(a, abs_sum, m, partials);
+  else k_bispec_sums<T, false><<<nblocks, 256, 0, s>>>(a, abs_sum, m, partials);
 }
 
 // delta = rho / mean - 1; FP32 data use 1 / mean as a float pair (hi + lo),
@@ -493,8 +543,7 @@ void launch_axpy(const T* x, const T* y, T* out, int64_t m, cudaStream_t s) {
   template void launch_axpy<T>(const T*, const T*, T*, int64_t, cudaStream_t);                                 \
   template void launch_sph_update<T>(const T*, T*, int64_t, double, double*, int, cudaStream_t); \
   template void launch_sum<T>(const T*, int64_t, bool, double*, int, cudaStream_t);            \
-  template void launch_product3_sum<T>(const T*, const T*, const T*, int64_t, double*, int,    \
-                                       cudaStream_t);                                          \
+  template void launch_bispec_sums<T>(T* const*, const double*, int64_t, double*, int, cudaStream_t);         \
   template void launch_density_contrast<T>(const T*, T*, int64_t, const double*, cudaStream_t); \
   template void launch_fill<T>(T*, int64_t, T, cudaStream_t);                                  \
   template void launch_sub_mean<T>(const T*, T*, int64_t, const double*, cudaStream_t);
