@@ -1192,7 +1192,7 @@ DGP_INST_XY(512)
 
 #define DGP_INST_X(T, N)                                                                            \
   template void launch_fft_x_op<T, N>(int, const vec2_t<T>*, const vec2_t<T>*, const FieldSet<T>&, int, \
-                                      const KParams&, double*, int, double, double, const vec2_t<T>*,   \
+                                      const KParams&, double*, int, int, int, const vec2_t<T>*,         \
                                       cudaStream_t, const int*, vec2_t<T>*);                             \
   template void launch_fft_x_adj<T, N>(int, const FieldSet<T>&, int, const FieldSet<T>&, const KParams&,  \
                                        const vec2_t<T>*, cudaStream_t);                                  \
