@@ -125,6 +125,46 @@ __device__ __forceinline__ void dft3(V& a, V& b, V& c) {
   c = cmake<V>(t.x - h * d.y, t.y + h * d.x);
 }
 
+// W_24^j = exp(-2 pi i j / 24) from the decimal expansions of cos(pi j / 12).
+__host__ __device__ constexpr double cos_pi12(int j) {
+  j = ((j % 24) + 24) % 24;
+  if (j > 12) j = 24 - j;
+  if (j > 6) return -cos_pi12(12 - j);
+  return j == 0 ? 1.0
+       : j == 1 ? 0.96592582628906828675
+       : j == 2 ? 0.86602540378443864676
+       : j == 3 ? 0.70710678118654752440
+       : j == 4 ? 0.5
+       : j == 5 ? 0.25881904510252076235
+       : 0.0;
+}
+template <typename V> __device__ __forceinline__ V twiddle24(int j) {
+  using S = decltype(V::x);
+  return cmake<V>((S)cos_pi12(j), (S)-cos_pi12(j - 6));
+}
+
+template <int R, int TWS, typename V>
+__device__ __forceinline__ void dft_regs(V (&v)[R], const V* __restrict__ tw);
+
+// R = 12 or 24 as two R/2-point DFTs of the even and odd elements.
+template <int R, typename V>
+__device__ __forceinline__ void dft_halves(V (&v)[R], const V* __restrict__ tw) {
+  V e[R / 2], o[R / 2];
+#pragma unroll
+  for (int i = 0; i < R / 2; ++i) {
+    e[i] = v[2 * i];
+    o[i] = v[2 * i + 1];
+  }
+  dft_regs<R / 2, 1>(e, tw);
+  dft_regs<R / 2, 1>(o, tw);
+#pragma unroll
+  for (int k = 0; k < R / 2; ++k) {
+    const V t = k == 0 ? o[k] : 4 * k == R ? cmake<V>(o[k].y, -o[k].x) : cmul(o[k], twiddle24<V>(24 / R * k));
+    v[k] = cadd(e[k], t);
+    v[k + R / 2] = csub(e[k], t);
+  }
+}
+
 // Forward DFT of the R values in v (natural order in and out): R = 3 directly,
 // R = 6 as two 3-point DFTs of the even and odd elements combined with
 // W_6^k = 1/2 - i h, -1/2 - i h (decimation in time), otherwise radix-2
@@ -147,6 +187,8 @@ __device__ __forceinline__ void dft_regs(V (&v)[R], const V* __restrict__ tw) {
     v[4] = csub(e1, t1);
     v[2] = cadd(e2, t2);
     v[5] = csub(e2, t2);
+  } else if constexpr (R == 12 || R == 24) {
+    dft_halves<R>(v, tw);
   } else {
     dft_regs_pow2<R>(v);
   }

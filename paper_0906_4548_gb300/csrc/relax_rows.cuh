@@ -1,4 +1,4 @@
-// The relaxation pass with every row transformed inside one warp (power-of-two meshes).
+// The relaxation pass with every row transformed inside one warp.
 // Included by relax_tma.cu, which holds the arithmetic policies, the TMA helpers and the host side.
 //
 // A row is a pencil of the tile transforms of tile_slots.cuh (N2 lanes of a warp; the transpose of a
@@ -22,8 +22,23 @@
 
 namespace dgp {
 
+// Split of a row: that of the other passes, except that 48 takes four lanes of 12 samples and 96 eight
+// lanes of 12 (rows of 3 or 6 lanes do not fill warps), with twiddles from the table of all W_N^t
+// instead of the phase table of the other split.  At 96 the 12 columns of the second stage take two
+// rounds of the 8 lanes, the second half empty, and D_new goes through shared memory to the lanes of
+// the forward transform.  (Four lanes of 24 samples need 128 registers and leave 8 warps per SM to a
+// single 96^3 mesh: 25 us against 22 for rows spread over the CTA.)
+template <int N> struct RowSplit {
+  static constexpr int N1 = Split<N>::N1, N2 = Split<N>::N2;
+  static constexpr bool PHASES = true;
+};
+template <> struct RowSplit<48> { static constexpr int N1 = 12, N2 = 4; static constexpr bool PHASES = false; };
+template <> struct RowSplit<96> { static constexpr int N1 = 12, N2 = 8; static constexpr bool PHASES = false; };
+
 template <int N> struct RowGeom {
-  static constexpr int N1 = Split<N>::N1, N2 = Split<N>::N2, Q = N1 / N2;
+  static constexpr int N1 = RowSplit<N>::N1, N2 = RowSplit<N>::N2, Q = (N1 + N2 - 1) / N2;
+  static constexpr bool EVEN = N1 % N2 == 0;  // every round of the second stage is full
+  static constexpr int PTS = Q * N2;          // values of a lane after it
   static constexpr int TY = 16, THREADS = TY * N2, WARPS = THREADS / 32;
   static constexpr int NK = N / 2 + 1;
   static constexpr int NBOX = (NK + 255) / 256;
@@ -38,52 +53,68 @@ template <int N> struct RowGeom {
   static constexpr int EXTRA = 16 + 4 * 8 * WARPS + 16 + 32;  // barriers, partials, mean, counters
   static constexpr size_t SMEM = 1024 + 2 * BUF + N * 8 + EXTRA;
   // 24 warps per SM at 80 registers
-  static constexpr int MINB = N <= 256 ? 768 / THREADS : 1;
-  static_assert(Q >= 1, "power-of-two split with N2 <= N1");
+  static constexpr int MINB = N == 512 ? 1 : 768 / THREADS;
 };
 
-// Real DFT of R values: X[0..R/2], X[0] and X[R/2] real.  Decimation in time.
+// W_R^k, R dividing 32 or 24
+template <int R> __device__ __forceinline__ float2 twiddle_r(int k) {
+  if constexpr (32 % R == 0) return twiddle_c<float2, R>(k);
+  else return twiddle24<float2>(24 / R * k);
+}
+
+// Real DFT of R values: X[0..R/2], X[0] and (R even) X[R/2] real.  Decimation in time.
 template <int R>
 __device__ __forceinline__ void rdft(const float (&x)[R], float2 (&X)[R / 2 + 1]) {
   if constexpr (R == 2) {
     X[0] = make_float2(x[0] + x[1], 0.f);
     X[1] = make_float2(x[0] - x[1], 0.f);
+  } else if constexpr (R == 3) {
+    const float h = 0.86602540378443864676f, s = x[1] + x[2];
+    X[0] = make_float2(x[0] + s, 0.f);
+    X[1] = make_float2(x[0] - 0.5f * s, -h * (x[1] - x[2]));
   } else {
-    float e[R / 2], o[R / 2];
+    constexpr int H = R / 2;
+    float e[H], o[H];
 #pragma unroll
-    for (int i = 0; i < R / 2; ++i) {
+    for (int i = 0; i < H; ++i) {
       e[i] = x[2 * i];
       o[i] = x[2 * i + 1];
     }
-    float2 E[R / 4 + 1], O[R / 4 + 1];
-    rdft<R / 2>(e, E);
-    rdft<R / 2>(o, O);
+    float2 E[H / 2 + 1], O[H / 2 + 1];
+    rdft<H>(e, E);
+    rdft<H>(o, O);
     X[0] = make_float2(E[0].x + O[0].x, 0.f);
-    X[R / 2] = make_float2(E[0].x - O[0].x, 0.f);
+    X[H] = make_float2(E[0].x - O[0].x, 0.f);
 #pragma unroll
-    for (int k = 1; k < R / 4; ++k) {
+    for (int k = 1; 2 * k < H; ++k) {
       float2 t;
       if (8 * k == R) {
         const float c = 0.70710678118654752440f;
         t = make_float2((O[k].x + O[k].y) * c, (O[k].y - O[k].x) * c);
       } else {
-        t = cmul(O[k], twiddle_c<float2, R>(k));
+        t = cmul(O[k], twiddle_r<R>(k));
       }
       X[k] = cadd(E[k], t);
-      X[R / 2 - k] = cconj(csub(E[k], t));
+      X[H - k] = cconj(csub(E[k], t));
     }
-    X[R / 4] = make_float2(E[R / 4].x, -O[R / 4].x);
+    if constexpr (H % 2 == 0) X[H / 2] = make_float2(E[H / 2].x, -O[H / 2].x);
   }
 }
 
-// the row's slots: those from N / 2 on are in the second tile
-template <int N> using RowSlots = TileSlots<N, RowGeom<N>::FIELD - (N / 2) * 128>;
+// W_N^{k1 c} of the four-step split from the table in shared memory
+template <int N> __device__ __forceinline__ float2 row_phase(const float2* s_tw, int k1, int c) {
+  if constexpr (RowSplit<N>::PHASES) return s_tw[k1 * RowSplit<N>::N2 + c];
+  else return s_tw[k1 * c];
+}
 
-// Inverse z transform of the pair in buf: on return a[j1], b[j1] are the two fields at
-// z = c + N2 j1, j1 = q + Q k2.
+// the row's slots: those from N / 2 on are in the second tile
+template <int N> using RowSlots = TileSlots<RowGeom<N>::N1, RowGeom<N>::N2, RowGeom<N>::FIELD - (N / 2) * 128>;
+
+// Inverse z transform of the pair in buf: on return a[i], b[i] with i = q + Q k2 are the two fields at
+// z = k1 + N1 k2, k1 = c + N2 q (zero where k1 >= N1); z = c + N2 i when N1 is a multiple of N2.
 template <int N>
 __device__ __forceinline__ void row_pair_inverse(unsigned char* buf, const float2* s_tw, int r, int c,
-                                                 float (&a)[Split<N>::N1], float (&b)[Split<N>::N1]) {
+                                                 float (&a)[RowGeom<N>::PTS], float (&b)[RowGeom<N>::PTS]) {
   using G = RowGeom<N>;
   using S = RowSlots<N>;
   constexpr int N1 = G::N1, N2 = G::N2, Q = G::Q;
@@ -114,11 +145,16 @@ __device__ __forceinline__ void row_pair_inverse(unsigned char* buf, const float
     dft_regs<N1, N / N1>(v, s_tw);
 #pragma unroll
     for (int k1 = 0; k1 < N1; ++k1)
-      tile_at(buf, S::by_col(off_d, k1)) = k1 == 0 ? v[k1] : cmul(v[k1], s_tw[k1 * N2 + c]);
+      tile_at(buf, S::by_col(off_d, k1)) = k1 == 0 ? v[k1] : cmul(v[k1], row_phase<N>(s_tw, k1, c));
   }
   __syncwarp();
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
+    if (!G::EVEN && c + N2 * q >= N1) {
+#pragma unroll
+      for (int k2 = 0; k2 < N2; ++k2) a[q + Q * k2] = b[q + Q * k2] = 0.f;
+      continue;
+    }
     const int base = S::by_row_base(c + N2 * q, r);
     float2 u[N2];
 #pragma unroll
@@ -136,7 +172,7 @@ __device__ __forceinline__ void row_pair_inverse(unsigned char* buf, const float
 // the first tile of buf in the tile layout (line kz, row r).
 template <int N>
 __device__ __forceinline__ void row_forward(unsigned char* buf, const float2* s_tw, int r, int c,
-                                            const float (&d)[Split<N>::N1]) {
+                                            const float (&d)[RowGeom<N>::N1]) {
   using G = RowGeom<N>;
   using S = RowSlots<N>;
   constexpr int N1 = G::N1, N2 = G::N2;
@@ -146,7 +182,7 @@ __device__ __forceinline__ void row_forward(unsigned char* buf, const float2* s_
     const int base = S::line(c, r);
 #pragma unroll
     for (int k1 = 0; k1 <= N1 / 2; ++k1) {
-      const float2 w = s_tw[k1 * N2 + c];
+      const float2 w = row_phase<N>(s_tw, k1, c);
       const float2 t = k1 == 0 ? V[0] : k1 == N1 / 2 ? make_float2(V[k1].x * w.x, V[k1].x * w.y) : cmul(V[k1], w);
       tile_at(buf, S::by_col(base, k1)) = t;
     }
@@ -229,7 +265,7 @@ __global__ void __launch_bounds__(RowGeom<N>::THREADS, RowGeom<N>::MINB)
     mp[1] = (float)(m - (double)mp[0]);
     s_cnt[0] = s_cnt[1] = s_cnt[2] = s_cnt[3] = 0;
   }
-  for (int i = tid; i < N; i += G::THREADS) s_tw[i] = g_tw[N + i];
+  for (int i = tid; i < N; i += G::THREADS) s_tw[i] = g_tw[(RowSplit<N>::PHASES ? N : 0) + i];
   __syncthreads();
   const double mean = s_mean[0];
   const float m_hi = reinterpret_cast<const float*>(s_mean + 1)[0];
@@ -260,17 +296,18 @@ __global__ void __launch_bounds__(RowGeom<N>::THREADS, RowGeom<N>::MINB)
   };
   auto gave_up = [&]() { return *reinterpret_cast<volatile int*>(&s_cnt[3]) != 0; };
 
-  Acc acc[N1];
-  float ra[N1], rb[N1];
+  constexpr int PTS = G::PTS, Q = G::Q;
+  Acc acc[PTS];
+  float ra[PTS], rb[PTS];
   wait(&bars[0], 0);
   row_pair_inverse<N>(buf0, s_tw, r, c, ra, rb);
 #pragma unroll
-  for (int i = 0; i < N1; ++i) AR::pair_a(acc[i], ra[i], rb[i]);
+  for (int i = 0; i < PTS; ++i) AR::pair_a(acc[i], ra[i], rb[i]);
   if (last_warp(0) && wl == 0 && !gave_up()) issue(buf0, 0, 1, &bars[0]);  // pair C, the diagonal
   wait(&bars[1], 0);
   row_pair_inverse<N>(buf1, s_tw, r, c, ra, rb);
 #pragma unroll
-  for (int i = 0; i < N1; ++i) AR::pair_b(acc[i], ra[i], rb[i], rp);
+  for (int i = 0; i < PTS; ++i) AR::pair_b(acc[i], ra[i], rb[i], rp);
   float* sD = reinterpret_cast<float*>(buf1);
   float* sS = sD + TY * ROWP;
   const int64_t rbase0 = ((int64_t)x * N + y0) * N;
@@ -286,10 +323,12 @@ __global__ void __launch_bounds__(RowGeom<N>::THREADS, RowGeom<N>::MINB)
   Sum rsum{};
   FP acc_d{0.f, 0.f};  // sum of D_new: its mean is removed next iteration
   float nbad = 0.f, nonfin = 0.f;
-  float* dst = args.Dnew + rbase0 + (int64_t)r * N + c;
+  float* dst = args.Dnew + rbase0 + (int64_t)r * N;
 #pragma unroll
-  for (int i = 0; i < N1; ++i) {
-    const int z = c + N2 * i;
+  for (int i = 0; i < PTS; ++i) {
+    const int k1 = c + N2 * (i % Q);
+    if (!G::EVEN && k1 >= N1) continue;
+    const int z = G::EVEN ? c + N2 * i : k1 + N1 * (i / Q);
     const PointOut o = AR::finish(acc[i], ra[i], rb[i], sD[r * ROWP + z], sS[r * ROWP + z], m_hi, m_lo, mean, rp,
                                   rsum, nonfin);
     float bpt = o.bp, dt = o.dt;
@@ -306,13 +345,21 @@ __global__ void __launch_bounds__(RowGeom<N>::THREADS, RowGeom<N>::MINB)
     } else {
       dn = 2.f * bpt / (rp.alpha_f + sqrtf(dt));
     }
-    dst[N2 * i] = dn;
-    ra[i] = dn;
+    dst[z] = dn;
+    if constexpr (G::EVEN) ra[i] = dn;
+    else sD[r * ROWP + z] = dn;
     if constexpr (std::is_same<AR, RxF32>::value) acc_d.hi += dn;
     else fp_acc(acc_d, FP{dn, 0.f});
   }
-  __syncwarp();  // the row's slots of buf0 are read
-  row_forward<N>(buf0, s_tw, r, c, ra);
+  __syncwarp();  // the row's slots of buf0 are read, its D_new is written
+  if constexpr (G::EVEN) {
+    row_forward<N>(buf0, s_tw, r, c, ra);
+  } else {
+    float d[N1];
+#pragma unroll
+    for (int j1 = 0; j1 < N1; ++j1) d[j1] = sD[r * ROWP + N2 * j1 + c];
+    row_forward<N>(buf0, s_tw, r, c, d);
+  }
   // ---- statistics: within a warp float pairs (FP64 for the FP64 policy), across warps FP64
   if constexpr (std::is_same<Sum, double>::value) {
     double v4[4] = {rsum, (double)acc_d.hi + (double)acc_d.lo, (double)nbad, (double)nonfin};

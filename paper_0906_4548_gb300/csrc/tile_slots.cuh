@@ -7,18 +7,19 @@
 // pencil).  Lane c does the N1-point transforms of column c and the N2-point transforms of rows
 // k1 = c, c + N2, ...; in between, value (k1, c) sits in line k1 N2 + (c ^ (k1 & 7)) of its own
 // pencil.  Both directions are free of bank conflicts for N2 >= 8, and no other warp touches the
-// pencil's slots, so a transform needs __syncwarp only.  Lines from N / 2 on may lie `FOLD` bytes
-// further (a second tile).
+// pencil's slots, so a transform needs __syncwarp only.  Lines from N / 2 on lie `FOLD` bytes further
+// (in a second tile).  When N1 is a multiple of N2, the values of lane c after the second
+// stage, k1 + N1 k2 with k1 = c mod N2, are again samples of its column.
 #pragma once
 
 #include "fft_core.cuh"
 
 namespace dgp {
 
-template <int N, int FOLD = 0> struct TileSlots {
-  static constexpr int N1 = Split<N>::N1, N2 = Split<N>::N2, Q = N1 / N2;
+template <int N1, int N2, int FOLD> struct TileSlots {
   static constexpr int M = N2 < 8 ? N2 - 1 : 7;
-  static_assert(N2 == 4 || N2 == 8 || N2 == 16, "power-of-two split");
+  static_assert(N2 == 4 || N2 == 8 || N2 == 16, "the lanes of a pencil divide a warp");
+  static_assert((N1 * N2) % 16 == 0 && N1 % 2 == 0, "whole swizzle periods in both halves");
   static __host__ __device__ constexpr int col(int k1) { return k1 * N2 * 128 + (k1 >= N1 / 2 ? FOLD : 0); }
   static __host__ __device__ constexpr int odd4(int k1) { return N2 == 4 ? (k1 & 1) << 6 : 0; }
   // byte offset of line l, pencil r (first tile)
