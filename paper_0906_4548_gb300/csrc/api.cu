@@ -361,6 +361,7 @@ class Engine : public EngineBase {
   SolveCtl* d_ctl = nullptr;    // stop-rule state of the running solve
   SolveCtl* h_ctl = nullptr;    // pinned host copy
   double* d_hist = nullptr;     // [max_iter + 1] normalised residuals of the running solve
+  double* h_hist = nullptr;     // pinned host copy, read with the verdict
   int last_stop_it = -1;        // last iteration examined by the previous solve
   double last_nl_a = -1.0;      // scale factor of the last nonlinear solve
   static constexpr int kPatience = 10;  // iterations without a new minimum before stopping
@@ -411,7 +412,7 @@ class Engine : public EngineBase {
     cudaFree(srt_key); cudaFree(srt_cell); cudaFree(srt_sums);
     cudaFree(aP); cudaFree(aF); cudaFree(aS); cudaFree(d_adj); cudaFree(aFb);
     for (int i = 0; i < 6; ++i) cudaFree(ap[i]);
-    cudaFree(d_ctl); cudaFree(d_hist); cudaFreeHost(h_ctl);
+    cudaFree(d_ctl); cudaFree(d_hist); cudaFreeHost(h_ctl); cudaFreeHost(h_hist);
     for (int j = 0; j < kCopyStreams; ++j)
       if (copy_streams[j]) cudaStreamDestroy(copy_streams[j]);
     for (int j = 0; j <= kCopyStreams; ++j)
@@ -456,6 +457,7 @@ class Engine : public EngineBase {
     if (cudaMalloc(&d_ctl, sizeof(SolveCtl)) != cudaSuccess) return DGP_E_NOMEM;
     if (cudaMallocHost(&h_ctl, sizeof(SolveCtl)) != cudaSuccess) return DGP_E_NOMEM;
     if (cudaMalloc(&d_hist, sizeof(double) * ((size_t)p.max_iter + 1)) != cudaSuccess) return DGP_E_NOMEM;
+    if (cudaMallocHost(&h_hist, sizeof(double) * ((size_t)p.max_iter + 1)) != cudaSuccess) return DGP_E_NOMEM;
     pk_blocks = x_pass_blocks<T, N>();
     if (cudaMalloc(&pk_partials, sizeof(double) * 4 * (N / 2) * (size_t)pk_blocks) != cudaSuccess) return DGP_E_NOMEM;
     if (cudaMalloc(&d_pk, sizeof(double) * 4 * (N / 2)) != cudaSuccess) return DGP_E_NOMEM;
@@ -800,6 +802,8 @@ class Engine : public EngineBase {
           }
         }
         DGP_CUDA(cudaMemcpyAsync(h_ctl, d_ctl, sizeof(SolveCtl), cudaMemcpyDeviceToHost, stream));
+        DGP_CUDA(cudaMemcpyAsync(h_hist, d_hist, sizeof(double) * std::min(it, p.max_iter + 1), cudaMemcpyDeviceToHost,
+                                 stream));
         DGP_CUDA(wait_stream());
         if (h_ctl->done || it > p.max_iter) break;
         chunk = kChunk;
@@ -808,9 +812,7 @@ class Engine : public EngineBase {
       if (!st.done) return DGP_E_STATE;  // the controller stops at it = max_iter at the latest
       const int s_it = st.stop_it;
       credit(s_it + 1, s_it);
-      history.assign(s_it + 1, 0.0);
-      DGP_CUDA(cudaMemcpyAsync(history.data(), d_hist, sizeof(double) * (s_it + 1), cudaMemcpyDeviceToHost, stream));
-      DGP_CUDA(wait_stream());
+      history.assign(h_hist, h_hist + s_it + 1);
       if (st.status == CTL_FAULT) return DGP_E_TIMEOUT;
       if (st.status == CTL_NONFINITE) return DGP_E_NONFINITE;
       last_stop_it = s_it;
@@ -1192,8 +1194,9 @@ class Engine : public EngineBase {
       pf.run(KK_Z_R2C, nR + nS, st, [&] { launch_fft_z_r2c_batch<T, N>(in, out, pro, n, tw, st); });
       if (!plane) pf.run(KK_Y, 2 * nS, st, [&] { launch_fft_y_batch<T, N>(f, nullptr, nullptr, n, 1, false, tw, st, yt); });
     }
-    for (int k = 0; k < n; ++k)
-      if (cudaMemsetAsync(S[k]->d_ctl, 0, sizeof(SolveCtl), st) != cudaSuccess) return DGP_E_CUDA;
+    VerdictBatch vb;
+    for (int k = 0; k < n; ++k) vb.m[k] = {S[k]->d_ctl, S[k]->d_hist, S[k]->h_ctl, S[k]->h_hist, S[k]->p.max_iter + 1};
+    launch_clear_verdicts(vb, n, st);
     int rc;
     if ((rc = check())) return rc;
     // one iteration of the members in ks
@@ -1323,9 +1326,9 @@ class Engine : public EngineBase {
           ++it;
         }
       }
-      for (int k = 0; k < n; ++k)
-        if (cudaMemcpyAsync(S[k]->h_ctl, S[k]->d_ctl, sizeof(SolveCtl), cudaMemcpyDeviceToHost, st) != cudaSuccess)
-          return DGP_E_CUDA;
+      // every member's verdict and residuals straight to pinned host memory, one launch
+      launch_fetch_verdicts(vb, n, it, st);
+      if ((rc = check())) return rc;
       if (e0->wait_stream() != cudaSuccess) return DGP_E_CUDA;
       bool done = true;
       for (int k = 0; k < n; ++k) done = done && S[k]->h_ctl->done;
@@ -1337,13 +1340,11 @@ class Engine : public EngineBase {
     for (int k = 0; k < n; ++k) {
       ctl[k] = *S[k]->h_ctl;
       if (!ctl[k].done) return DGP_E_STATE;
-      S[k]->history.assign(ctl[k].stop_it + 1, 0.0);
-      if (cudaMemcpyAsync(S[k]->history.data(), S[k]->d_hist, sizeof(double) * (ctl[k].stop_it + 1),
-                          cudaMemcpyDeviceToHost, st) != cudaSuccess)
-        return DGP_E_CUDA;
+      S[k]->history.assign(S[k]->h_hist, S[k]->h_hist + ctl[k].stop_it + 1);
     }
-    if (e0->wait_stream() != cudaSuccess) return DGP_E_CUDA;
     std::vector<V*> sDphi(n);
+    FieldSet<T> fy[kBatchMax];  // plane pass: accepted spectra still to be transformed along y
+    int ny = 0;
     for (int k = 0; k < n; ++k) {
       Engine* e = S[k];
       const SolveCtl& c = ctl[k];
@@ -1357,7 +1358,7 @@ class Engine : public EngineBase {
         sDphi[k] = spec_in(k, s_it);
         if (plane) {  // the accepted iterate's spectrum is transformed along z only
           V* f1[1] = {sDphi[k]};
-          pf.run(KK_Y, 2 * SB, st, [&] { launch_fft_y<T, N>(fs(f1, 1), 1, false, tw, st, nullptr, yt); });
+          fy[ny++] = fs(f1, 1);
         }
       } else {
         // an earlier iterate: replay the iterations that produced it for this member alone
@@ -1395,6 +1396,9 @@ class Engine : public EngineBase {
         inf.status = c.status == CTL_CONVERGED ? DGP_OK : DGP_E_NOT_CONVERGED;
       }
     }
+    if (ny)
+      pf.run(KK_Y, 2.0 * ny * SB, st,
+             [&] { launch_fft_y_batch<T, N>(fy, nullptr, nullptr, ny, 1, false, tw, st, yt); });
     // forces g = -grad phi (Eq. FullDGP1) of every member
     {
       XReal<T> xr[kBatchMax];
@@ -1412,8 +1416,7 @@ class Engine : public EngineBase {
       pf.run(KK_Z_C2R, 3.0 * (nS + nR), st, [&] { launch_fft_z_c2r_batch<T, N>(fi, fo, 3, n, tw, st); });
     }
     if ((rc = check())) return rc;
-    if (info && e0->wait_stream() != cudaSuccess) return DGP_E_CUDA;
-    return status;
+    return status;  // dgp_batch_step waits for the class's stream before it returns
   }
 
  public:

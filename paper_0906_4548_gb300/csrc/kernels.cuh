@@ -297,6 +297,19 @@ struct SolveCtl {
   double rbest, rprev, prev_nbad, last_bad;
   double eps, rnorm;  // <|S|> and the normalisation of the residual
 };
+// A class's stop-rule states: cleared before a solve, and fetched (with the residuals of the first
+// `iters` iterations, at most the member's array) into pinned host memory, one launch each.
+struct VerdictBatch {
+  struct {
+    SolveCtl* ctl;
+    const double* hist;
+    SolveCtl* h_ctl;
+    double* h_hist;
+    int hist_len;
+  } m[kBatchMax];
+};
+void launch_clear_verdicts(const VerdictBatch& b, int count, cudaStream_t s);
+void launch_fetch_verdicts(const VerdictBatch& b, int count, int iters, cudaStream_t s);
 // stats: [sum |R|, sum D_new, bad points, non-finite R] of the iteration
 // it = ctl->next_it (counted on the device, so the same launch serves every
 // iteration of a captured graph); abs_src_sum: sum |S| (read at it = 0);

@@ -173,6 +173,28 @@ void launch_control_batch(const YControl* ctl, const int* const* skip, int count
   k_control_batch<<<count, 256, 0, s>>>(b);
 }
 
+__global__ void __launch_bounds__(128) k_clear_verdicts(const __grid_constant__ VerdictBatch b) {
+  int* c = reinterpret_cast<int*>(b.m[blockIdx.x].ctl);
+  for (int i = threadIdx.x; i < (int)(sizeof(SolveCtl) / sizeof(int)); i += blockDim.x) c[i] = 0;
+}
+// Replaces two copies per member (32 for a class of 16, one of each pair to pageable memory).
+__global__ void __launch_bounds__(128) k_fetch_verdicts(const __grid_constant__ VerdictBatch b, int iters) {
+  const auto& m = b.m[blockIdx.x];
+  const int* c = reinterpret_cast<const int*>(m.ctl);
+  int* h = reinterpret_cast<int*>(m.h_ctl);
+  for (int i = threadIdx.x; i < (int)(sizeof(SolveCtl) / sizeof(int)); i += blockDim.x) h[i] = c[i];
+  const int n = iters < m.hist_len ? iters : m.hist_len;
+  for (int i = threadIdx.x; i < n; i += blockDim.x) m.h_hist[i] = m.hist[i];
+}
+void launch_clear_verdicts(const VerdictBatch& b, int count, cudaStream_t s) {
+  if (count < 1 || count > kBatchMax) return;
+  k_clear_verdicts<<<count, 128, 0, s>>>(b);
+}
+void launch_fetch_verdicts(const VerdictBatch& b, int count, int iters, cudaStream_t s) {
+  if (count < 1 || count > kBatchMax) return;
+  k_fetch_verdicts<<<count, 128, 0, s>>>(b, iters);
+}
+
 // The stop rules as a launch of their own (relax_control.cuh).
 __global__ void k_relax_control(SolveCtl* __restrict__ c, const double* __restrict__ stats,
                                 const double* __restrict__ abs_src_sum, double* __restrict__ hist,
