@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(XGeom<T, N>::THREADS, XGeom<T, N>::MIN_BLOCKS)
   // rows), then the shell sums of two halves of the columns, [2][NBS][nbins]
   constexpr int NBS = OP == XOP_PK_BRANE ? 4 : 3;  // sums per shell
   double* s_bins = reinterpret_cast<double*>(s_T + N * (TY + 1));
-  V* s_T2 = reinterpret_cast<V*>(s_inv);  // the Hessian op's second transpose buffer (N * TY)
+  V* s_T2 = reinterpret_cast<V*>(s_inv);  // or, for operations without the tables, a second transpose buffer (N * TY)
   load_twiddles(s_tw, g_tw, N);
   const int yl = threadIdx.x % TY;
   const int lane = threadIdx.x / TY;
@@ -381,9 +381,10 @@ __global__ void __launch_bounds__(XGeom<T, N>::THREADS, XGeom<T, N>::MIN_BLOCKS)
   }
 
   constexpr int NT = XGeom<T, N>::THREADS;
+  constexpr bool TABLES = OP == XOP_SOURCE || OP == XOP_SOURCE_LIN || OP == XOP_ADJ_PHI || OP == XOP_ADJ_COMBINE;
   const T inv_m = kc<T>(kp.inv_m, kp.inv_m_f);
 #pragma unroll
-  for (int k2 = 0; k2 < N2 && OP != XOP_HESSIAN && OP != XOP_PHI_FORCE; ++k2) {
+  for (int k2 = 0; k2 < N2 && TABLES; ++k2) {
     const int nx = signed_index(lane + N1 * k2, N);
     const int n2 = nx * nx + ny * ny + nz * nz;
     T inv = (T)0, ikb = (T)0;
@@ -498,11 +499,11 @@ __global__ void __launch_bounds__(XGeom<T, N>::THREADS, XGeom<T, N>::MIN_BLOCKS)
         const int n2 = nx * nx + ny * ny + nz * nz;
         Y[k2] = cmake<V>((T)0, (T)0);
         if (n2 != 0) {
-          const T kmag = kf * sqrt((T)n2);
           T m;
           if (OP == XOP_ZEL_ADJ) {
-            m = (T)-1 / (kmag * kmag);
+            m = (T)-1 / (kf * kf * (T)n2);
           } else {
+            const T kmag = kf * sqrt((T)n2);
             const T ikb = s_ikb[k2 * NT + threadIdx.x];
             const T pref = -kc<T>(kp.aE * kp.aE, kp.aE2_f) / (kmag * kmag);
             const T den = (T)1 + ikb * kc<T>(1.0 / kp.eta, kp.inv_eta_f);
@@ -650,26 +651,27 @@ __global__ void __launch_bounds__(XGeom<T, N>::THREADS, XGeom<T, N>::MIN_BLOCKS)
     return;
   }
   if (OP == XOP_ZEL) {
-    const T inv_m = kc<T>(kp.inv_m, kp.inv_m_f);
+    // i k_j / k^2 = i n_j / (k_f n^2): the scale once, then n_j per output; the outputs alternate
+    // between two transpose buffers
+#pragma unroll
+    for (int k2 = 0; k2 < N2; ++k2) {
+      const int nx = signed_index(lane + N1 * k2, N);
+      const int n2 = nx * nx + ny * ny + nz * nz;
+      X0[k2] = cscale(X0[k2], n2 != 0 ? inv_m / (kf * (T)n2) : (T)0);
+    }
 #pragma unroll 1
     for (int o = 0; o < 3; ++o) {
-      const int nfix = o == 1 ? ny : nz;
+      const T fix = (T)(o == 1 ? ny : nz);
       const bool nyq_fix = o == 1 ? nyq_y : nyq_z;
       V Y[N2];
 #pragma unroll
       for (int k2 = 0; k2 < N2; ++k2) {
         const int kx = lane + N1 * k2;
-        const int nx = signed_index(kx, N);
-        const int n2 = nx * nx + ny * ny + nz * nz;
         const bool nyq = o == 0 ? kx == N / 2 : nyq_fix;
-        Y[k2] = cmake<V>((T)0, (T)0);
-        if (n2 != 0 && !nyq) {
-          const T ki = kf * (T)(o == 0 ? nx : nfix);
-          const T m = ki / (kf * kf * (T)n2) * inv_m;
-          Y[k2] = cmake<V>(-m * X0[k2].y, m * X0[k2].x);  // (i k_j / k^2) X
-        }
+        const T m = nyq ? (T)0 : (o == 0 ? (T)signed_index(kx, N) : fix);
+        Y[k2] = cmake<V>(-m * X0[k2].y, m * X0[k2].x);
       }
-      x_inverse<T, N>(Y, args.out.p[o], kz, ky0, lane, yl, s_T, s_tw);
+      x_inverse<T, N, false>(Y, args.out.p[o], kz, ky0, lane, yl, (o & 1) ? s_T2 : s_T, s_tw);
     }
     return;
   }

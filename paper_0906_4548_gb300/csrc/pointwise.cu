@@ -710,11 +710,37 @@ void launch_gather_kick_batch(const GatherArgs* a, int count, cudaStream_t s) {
   k_gather_kick_batch<<<dim3((unsigned)blocks, (unsigned)count), 256, 0, s>>>(b);
 }
 
+// four consecutive values, moved at once when the pointers allow it
+template <typename T> __device__ __forceinline__ void load4(const T* p, bool vec, T (&v)[4]) {
+  if constexpr (sizeof(T) == 4) {
+    if (vec) {
+      const float4 q = *reinterpret_cast<const float4*>(p);
+      v[0] = q.x; v[1] = q.y; v[2] = q.z; v[3] = q.w;
+      return;
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) v[j] = p[j];
+}
+template <typename T> __device__ __forceinline__ void store4(T* p, bool vec, const T (&v)[4]) {
+  if constexpr (sizeof(T) == 4) {
+    if (vec) {
+      *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+      return;
+    }
+  }
+#pragma unroll
+  for (int j = 0; j < 4; ++j) p[j] = v[j];
+}
+
+// A thread takes four points of a row (meshes have a multiple of 16 points a side), so the lattice
+// index costs two 32-bit divisions per four particles and the 9 fields move as 16-byte accesses.
 template <typename T>
-__global__ void k_zel_particles(const T* __restrict__ p0, const T* __restrict__ p1, const T* __restrict__ p2, T vf,
-                                CicParams cp, T* __restrict__ x, T* __restrict__ y, T* __restrict__ z,
-                                T* __restrict__ px, T* __restrict__ py, T* __restrict__ pz) {
-  const int64_t n = cp.n, m = n * n * n;
+__global__ void __launch_bounds__(256) k_zel_particles(const T* __restrict__ p0, const T* __restrict__ p1,
+                                                       const T* __restrict__ p2, T vf, CicParams cp, bool vec,
+                                                       T* __restrict__ x, T* __restrict__ y, T* __restrict__ z,
+                                                       T* __restrict__ px, T* __restrict__ py, T* __restrict__ pz) {
+  const unsigned n = (unsigned)cp.n, m4 = n * n * (n / 4);
   T box, inv_box;
   if constexpr (sizeof(T) == 8) {
     box = cp.box;
@@ -724,37 +750,78 @@ __global__ void k_zel_particles(const T* __restrict__ p0, const T* __restrict__ 
     inv_box = cp.inv_box_f;
   }
   const T d = box / (T)n;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t ix = i / (n * n), iy = (i / n) % n, iz = i % n;
-    x[i] = wrap_periodic((T)ix * d + p0[i], box, inv_box);
-    y[i] = wrap_periodic((T)iy * d + p1[i], box, inv_box);
-    z[i] = wrap_periodic((T)iz * d + p2[i], box, inv_box);
-    px[i] = vf * p0[i];
-    py[i] = vf * p1[i];
-    pz[i] = vf * p2[i];
+  for (unsigned q = blockIdx.x * blockDim.x + threadIdx.x; q < m4; q += gridDim.x * blockDim.x) {
+    const unsigned row = q / (n / 4), iz = (q - row * (n / 4)) * 4, ix = row / n, iy = row - ix * n;
+    const int64_t i = (int64_t)q * 4;
+    T a[4], o[4];
+    load4(p0 + i, vec, a);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) o[j] = wrap_periodic((T)ix * d + a[j], box, inv_box);
+    store4(x + i, vec, o);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) o[j] = vf * a[j];
+    store4(px + i, vec, o);
+    load4(p1 + i, vec, a);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) o[j] = wrap_periodic((T)iy * d + a[j], box, inv_box);
+    store4(y + i, vec, o);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) o[j] = vf * a[j];
+    store4(py + i, vec, o);
+    load4(p2 + i, vec, a);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) o[j] = wrap_periodic((T)(iz + j) * d + a[j], box, inv_box);
+    store4(z + i, vec, o);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) o[j] = vf * a[j];
+    store4(pz + i, vec, o);
   }
 }
 
 template <typename T>
-__global__ void k_zel_cot(const T* __restrict__ xb, const T* __restrict__ yb, const T* __restrict__ zb,
-                          const T* __restrict__ pxb, const T* __restrict__ pyb, const T* __restrict__ pzb, T vf,
-                          int64_t m, T* __restrict__ o0, T* __restrict__ o1, T* __restrict__ o2) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-    o0[i] = xb[i] + vf * pxb[i];
-    o1[i] = yb[i] + vf * pyb[i];
-    o2[i] = zb[i] + vf * pzb[i];
+__global__ void __launch_bounds__(256) k_zel_cot(const T* __restrict__ xb, const T* __restrict__ yb,
+                                                 const T* __restrict__ zb, const T* __restrict__ pxb,
+                                                 const T* __restrict__ pyb, const T* __restrict__ pzb, T vf,
+                                                 int64_t m, bool vec, T* __restrict__ o0, T* __restrict__ o1,
+                                                 T* __restrict__ o2) {
+  for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < m / 4; q += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = 4 * q;
+    T a[4], b[4];
+    load4(xb + i, vec, a);
+    load4(pxb + i, vec, b);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) a[j] += vf * b[j];
+    store4(o0 + i, vec, a);
+    load4(yb + i, vec, a);
+    load4(pyb + i, vec, b);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) a[j] += vf * b[j];
+    store4(o1 + i, vec, a);
+    load4(zb + i, vec, a);
+    load4(pzb + i, vec, b);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) a[j] += vf * b[j];
+    store4(o2 + i, vec, a);
   }
+}
+
+static bool aligned16(const void* const* p, int n) {
+  for (int i = 0; i < n; ++i)
+    if (reinterpret_cast<uintptr_t>(p[i]) & 15) return false;
+  return true;
 }
 
 template <typename T>
 void launch_zel_particles(T* const* psi, double vf, CicParams cp, T* const* out, cudaStream_t s) {
-  k_zel_particles<T><<<num_sms() * 4, 256, 0, s>>>(psi[0], psi[1], psi[2], (T)vf, cp, out[0], out[1], out[2],
-                                                   out[3], out[4], out[5]);
+  const void* ptr[9] = {psi[0], psi[1], psi[2], out[0], out[1], out[2], out[3], out[4], out[5]};
+  k_zel_particles<T><<<num_sms() * 8, 256, 0, s>>>(psi[0], psi[1], psi[2], (T)vf, cp, aligned16(ptr, 9), out[0],
+                                                   out[1], out[2], out[3], out[4], out[5]);
 }
 template <typename T>
 void launch_zel_cot(T* const* cot, double vf, int64_t m, T* const* psibar, cudaStream_t s) {
-  k_zel_cot<T><<<num_sms() * 4, 256, 0, s>>>(cot[0], cot[1], cot[2], cot[3], cot[4], cot[5], (T)vf, m, psibar[0],
-                                             psibar[1], psibar[2]);
+  const void* ptr[9] = {cot[0], cot[1], cot[2], cot[3], cot[4], cot[5], psibar[0], psibar[1], psibar[2]};
+  k_zel_cot<T><<<num_sms() * 8, 256, 0, s>>>(cot[0], cot[1], cot[2], cot[3], cot[4], cot[5], (T)vf, m,
+                                             aligned16(ptr, 9), psibar[0], psibar[1], psibar[2]);
 }
 
 #define DGP_INST_P(T)                                                                              \
