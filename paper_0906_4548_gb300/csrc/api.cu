@@ -388,9 +388,9 @@ class Engine : public EngineBase {
   int* srt_sums = nullptr;
   int64_t nsteps = 0;           // pm_step calls since init / reset
   // adjoint workspace (allocated on the first dgp_solve_adjoint)
-  T* aP = nullptr;              // [7][M]: H_f(D) lam for six pairs, then lam
+  T* aP = nullptr;              // [M]: lam
   T* aF = nullptr;              // [4][M]: u, Q, Dbar, A phibar
-  V* aS = nullptr;              // [7][SPEC]
+  V* aS = nullptr;              // [6][SPEC]
   double* d_adj = nullptr;      // [12]: sum u, sum r, sum 1/diag, nonpositive diag, sum |res|, sum |g|,
                                 // then the r_c terms: phibar and lam contractions, F . fbar, a dot product
   bool delta_nl = false;        // sDelta holds the spectrum of the last nonlinear solve's delta
@@ -1627,12 +1627,12 @@ class Engine : public EngineBase {
     if (p.gravity != DGP_GRAVITY_NL) return DGP_E_INVALID;
     if (wcur < 0 || !(last_nl_a > 0.0)) return DGP_E_STATE;
     if (rcbar && !delta_nl) return DGP_E_STATE;  // the r_c terms need that solve's delta
-    if (!aP && cudaMalloc(&aP, sizeof(T) * 7 * M) != cudaSuccess) { aP = nullptr; return DGP_E_NOMEM; }
+    if (!aP && cudaMalloc(&aP, sizeof(T) * M) != cudaSuccess) { aP = nullptr; return DGP_E_NOMEM; }
     if (!aF && cudaMalloc(&aF, sizeof(T) * 4 * M) != cudaSuccess) { aF = nullptr; return DGP_E_NOMEM; }
-    if (!aS && cudaMalloc(&aS, sizeof(V) * 7 * SPEC) != cudaSuccess) { aS = nullptr; return DGP_E_NOMEM; }
+    if (!aS && cudaMalloc(&aS, sizeof(V) * 6 * SPEC) != cudaSuccess) { aS = nullptr; return DGP_E_NOMEM; }
     if (!adj_scalars()) return DGP_E_NOMEM;
     int rc;
-    T* const lam = aP + 6 * M;
+    T* const lam = aP;
     T* const aU = aF;
     T* const aQ = aF + M;
     T* const aG = aF + 2 * M;
@@ -1642,7 +1642,7 @@ class Engine : public EngineBase {
     const ZPrologue none{nullptr, 0.0, 0};
     // cotangent spectra -> Dbar = B phibar_tot and A phibar_tot (real fields)
     FieldSet<T> in;
-    for (int i = 0; i < kMaxFields; ++i) in.p[i] = i < 7 ? aS + i * SPEC : nullptr;
+    for (int i = 0; i < kMaxFields; ++i) in.p[i] = i < 6 ? aS + i * SPEC : nullptr;
     int mask = 0;
     if (phibar) {
       if ((rc = forward_zy((const T*)phibar, in.p[0], none))) return rc;
@@ -1694,10 +1694,10 @@ class Engine : public EngineBase {
     const double gnorm = hs[5] > 0.0 ? hs[5] : 1.0;
     // lam_0 from rest = 0, then the w-split iteration
     DGP_CUDA(cudaMemsetAsync(lam, 0, sizeof(T) * M, stream));
-    DGP_CUDA(cudaMemsetAsync(aQ, 0, sizeof(T) * M, stream));
-    auto update = [&]() -> int {
-      prof.run(KK_RELAX, 6 * RB, stream, [&] {
-        launch_adj_update_a<T>(lam, rD[wcur], dsum, aG, aQ, aU, M, alpha, w, partials, nblocks, stream);
+    T* h5[5] = {rH[0], rH[1], rH[2], rH[3], rH[4]};
+    auto update = [&](const T* q) -> int {
+      prof.run(KK_RELAX, (q ? 7 : 3) * RB, stream, [&] {
+        launch_adj_update_a<T>(lam, rD[wcur], dsum, aG, q, h5, aU, M, alpha, w, partials, nblocks, stream);
       });
       prof.run(KK_REDUCE, 16.0 * nblocks, stream, [&] { launch_finalize(partials, nblocks, 2, d_adj, stream); });
       prof.run(KK_RELAX, 4 * RB, stream, [&] {
@@ -1707,30 +1707,24 @@ class Engine : public EngineBase {
       DGP_CHECK_LAUNCH();
       return DGP_OK;
     };
-    if ((rc = update())) return rc;
+    if ((rc = update(nullptr))) return rc;
     history.clear();
     dgp_solve_info inf;
     memset(&inf, 0, sizeof(inf));
     inf.eps = hs[5] / (double)M;
     bool converged = false;
-    T* h5[5] = {rH[0], rH[1], rH[2], rH[3], rH[4]};
-    FieldSet<T> aspec;
-    for (int i = 0; i < kMaxFields; ++i) aspec.p[i] = i < 7 ? aS + i * SPEC : nullptr;
     int it = 0;
     for (; it <= p.max_iter; ++it) {
-      prof.run(KK_MISC, 7 * RB, stream,
-               [&] { launch_adj_products<T>(lam, rD[wcur], dsum, h5, aP, M, stream); });
-      prof.run(KK_Z_R2C, 7 * (RB + SB), stream,
-               [&] { launch_fft_z_r2c<T, N>(aP, M, aS, SPEC, 7, none, tw, stream); });
-      prof.run(KK_Y, 14 * SB, stream, [&] { launch_fft_y<T, N>(aspec, 7, false, tw, stream, nullptr, y_threads); });
-      prof.run(KK_X_OTHER, 8 * SB, stream,
-               [&] { launch_fft_x_adj<T, N>(XOP_ADJ_COMBINE, aspec, 0x7f, fs(s6, 1), kp, tw, stream); });
+      prof.run(KK_Z_R2C, 7 * RB + 6 * SB, stream,
+               [&] { launch_adj_products_z<T, N>(lam, rD[wcur], dsum, h5, in.p, tw, stream); });
+      prof.run(KK_Y, 12 * SB, stream, [&] { launch_fft_y<T, N>(in, 6, false, tw, stream, nullptr, y_threads); });
+      prof.run(KK_X_OTHER, 7 * SB, stream,
+               [&] { launch_fft_x_adj<T, N>(XOP_ADJ_COMBINE, in, 0x3f, fs(s6, 1), kp, tw, stream); });
       T* qo[1] = {aQ};
       if ((rc = inverse_yz(s6, qo, 1))) return rc;
-      if ((rc = update())) return rc;
-      DGP_CUDA(cudaMemcpyAsync(hs, d_adj + 4, sizeof(double), cudaMemcpyDeviceToHost, stream));
-      DGP_CUDA(wait_stream());
-      const double r = hs[0] / gnorm;  // projected residual of the iterate before this update
+      if ((rc = update(aQ))) return rc;
+      if ((rc = fetch(d_adj + 4, 1))) return rc;
+      const double r = h_stats[0] / gnorm;  // projected residual of the iterate before this update
       history.push_back(r);
       if (!isfinite(r)) return DGP_E_NONFINITE;
       if (r < tol) {
@@ -2068,7 +2062,7 @@ static void workspace_bytes(int max_iter, int64_t np, dgp_workspace* w) {
             sizeof(double) * ((size_t)max_iter + 1) + sizeof(double) * 4 * (N / 2) * (size_t)x_pass_blocks<T, N>() +
             sizeof(double) * 4 * (N / 2) + sizeof(V) * 3 * N;
   w->sort = sizeof(int) * 3 * M + sizeof(int) * (size_t)sort_scan_blocks((int64_t)M) + (sizeof(int) + 6 * sizeof(T)) * pn;
-  w->adjoint = sizeof(T) * (7 + 4 + 3) * M + sizeof(V) * 7 * SPEC + sizeof(double) * 12 + 6 * sizeof(T) * pn;
+  w->adjoint = sizeof(T) * (1 + 4 + 3) * M + sizeof(V) * 6 * SPEC + sizeof(double) * 12 + 6 * sizeof(T) * pn;
   w->host_step = 6 * sizeof(T) * pn;
 }
 

@@ -525,12 +525,12 @@ __global__ void __launch_bounds__(XGeom<T, N>::THREADS, XGeom<T, N>::MIN_BLOCKS)
 #pragma unroll
     for (int k2 = 0; k2 < N2; ++k2) acc[k2] = cmake<V>((T)0, (T)0);
 #pragma unroll 1
-    for (int f = 0; f < 7; ++f) {
+    for (int f = 0; f < 6; ++f) {
       x_forward<T, N>(args.in.p[f], kz, ky0, lane, yl, s_T, s_tw, X0);
-      // pair (a, b) of input f: xx, yy, zz, xy, xz, yz; weight -2 (diagonal) or -4 (twice off-diagonal)
-      const int ca = f == 0 || f == 3 || f == 4 ? 0 : (f == 1 || f == 5 ? 1 : 2);
-      const int cb = f == 0 ? 0 : (f == 1 || f == 3 ? 1 : 2);
-      const T wgt = f < 3 ? (T)-2 : (T)-4;
+      // pair (a, b) of input f: yy, zz, xy, xz, yz; weight -2 (diagonal) or -4 (twice off-diagonal)
+      const int ca = f == 2 || f == 3 ? 0 : (f == 0 || f == 4 ? 1 : 2);
+      const int cb = f == 0 || f == 2 ? 1 : 2;
+      const T wgt = f < 2 ? (T)-2 : (T)-4;
       const T fa_fix = ca == 1 ? fy : fz, fb_fix = cb == 1 ? fy : fz;
       const bool nyq_fix = (ca != 0 && (ca == 1 ? nyq_y : nyq_z)) || (cb != 0 && (cb == 1 ? nyq_y : nyq_z));
 #pragma unroll
@@ -539,7 +539,7 @@ __global__ void __launch_bounds__(XGeom<T, N>::THREADS, XGeom<T, N>::MIN_BLOCKS)
         const T fx = (T)signed_index(kx, N);
         const T inv_n2 = s_inv[k2 * NT + threadIdx.x];
         T m;
-        if (f == 6) {
+        if (f == 5) {
           m = -kc<T>(kp.c2, kp.c2_f) * s_ikb[k2 * NT + threadIdx.x];  // c2 N = c2 (-1/kbar)
         } else {
           T prod = (ca == 0 ? fx : fa_fix) * (cb == 0 ? fx : fb_fix);

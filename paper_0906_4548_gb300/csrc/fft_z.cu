@@ -283,10 +283,120 @@ void launch_fft_z_c2r_batch(const FieldSet<T>* in, const FieldSet<T>* out, int n
   k_fft_z_c2r<T, N, kBatchMax><<<grid, G::THREADS, smem, s>>>(zb, nfields, tw);
 }
 
+// ---------------------------------------------------------------------------
+// Forward z pass of the adjoint relaxation with its products formed on the way in: the half spectra of
+// the six fields (H_yy - H_xx) lam, (H_zz - H_xx) lam, H_xy lam, H_xz lam, H_yz lam and lam, for H_ij the
+// real second derivatives of the accepted D (H_xx = D - <D> - H_yy - H_zz).  A CTA owns TY rows; two of
+// the fields of a row are packed into one complex pencil, three pencils one after another.  Reads 7
+// fields and writes 6 half spectra; as separate passes the products were written and read back
+// (13 fields more) and the three diagonal pairs took a transform each.
+template <typename T, int N> struct AZGeom {
+  static constexpr int N1 = Split<N>::N1, N2 = Split<N>::N2;
+  static constexpr int TY = sizeof(T) == 4 ? 16 : 8;
+  static constexpr int THREADS = TY * N1;
+  static constexpr int RS0 = N1 * (N2 + 1);
+  static constexpr int RS = N2 < N1 ? RS0 + ((N2 - RS0 % 16) % 16 + 16) % 16 : RS0;  // see relax_rows
+  static constexpr size_t SMEM = sizeof(vec2_t<T>) * (N + TY * RS + (size_t)N * (TY + 1));
+};
+template <typename T> struct AdjZArgs {
+  const T* lam;
+  const T* D;
+  const double* dsum;
+  const T* h[5];  // H_yy, H_zz, H_xy, H_xz, H_yz
+  vec2_t<T>* out[6];
+};
+
+template <typename T, int N>
+__global__ void __launch_bounds__(AZGeom<T, N>::THREADS, AZGeom<T, N>::THREADS <= 256 ? 2 : 1)
+    k_adj_products_z(const __grid_constant__ AdjZArgs<T> a, const vec2_t<T>* __restrict__ g_tw) {
+  using V = vec2_t<T>;
+  using G = AZGeom<T, N>;
+  constexpr int N1 = G::N1, N2 = G::N2, TY = G::TY, NK = N / 2 + 1;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  V* s_tw = reinterpret_cast<V*>(smem_raw);  // the phase table
+  V* s_T = s_tw + N;
+  V* s_Z = s_T + TY * G::RS;
+  __shared__ T s_mean;
+  if (threadIdx.x == 0) s_mean = (T)(a.dsum[0] / ((double)N * N * N));
+  for (int i = threadIdx.x; i < N; i += G::THREADS) s_tw[i] = g_tw[N + i];
+  const int lane = threadIdx.x % N1, row = threadIdx.x / N1;
+  const int r1 = threadIdx.x / N2, c1 = threadIdx.x % N2;
+  const bool act1 = N2 == N1 || threadIdx.x < TY * N2;
+  const int x = blockIdx.y, y0 = blockIdx.x * TY;
+  const int64_t base = ((int64_t)x * N + y0 + r1) * N + c1;
+  T lam[N1];
+  if (act1) {
+#pragma unroll
+    for (int j1 = 0; j1 < N1; ++j1) lam[j1] = a.lam[base + N2 * j1];
+  }
+  __syncthreads();
+  const T mean = s_mean;
+#pragma unroll 1
+  for (int p = 0; p < 3; ++p) {
+    if (act1) {
+      V v[N1];
+      if (p == 0) {
+#pragma unroll
+        for (int j1 = 0; j1 < N1; ++j1) {
+          const int64_t i = base + N2 * j1;
+          const T yy = a.h[0][i], zz = a.h[1][i], xx = (a.D[i] - mean) - yy - zz;
+          v[j1] = cmake<V>((yy - xx) * lam[j1], (zz - xx) * lam[j1]);
+        }
+      } else if (p == 1) {
+#pragma unroll
+        for (int j1 = 0; j1 < N1; ++j1) {
+          const int64_t i = base + N2 * j1;
+          v[j1] = cmake<V>(a.h[2][i] * lam[j1], a.h[3][i] * lam[j1]);
+        }
+      } else {
+#pragma unroll
+        for (int j1 = 0; j1 < N1; ++j1) v[j1] = cmake<V>(a.h[4][base + N2 * j1] * lam[j1], lam[j1]);
+      }
+      dft_regs<N1, N / N1>(v, s_tw);
+#pragma unroll
+      for (int k1 = 0; k1 < N1; ++k1)
+        s_T[r1 * G::RS + k1 * (N2 + 1) + c1] = k1 == 0 ? v[k1] : cmul(v[k1], s_tw[k1 * N2 + c1]);
+    }
+    __syncthreads();
+    {
+      V u[N2];
+#pragma unroll
+      for (int j2 = 0; j2 < N2; ++j2) u[j2] = s_T[row * G::RS + lane * (N2 + 1) + j2];
+      dft_regs<N2, N / N2>(u, s_tw);
+#pragma unroll
+      for (int k2 = 0; k2 < N2; ++k2) s_Z[(lane + N1 * k2) * (TY + 1) + row] = u[k2];
+    }
+    __syncthreads();
+    V* A = a.out[2 * p];
+    V* B = a.out[2 * p + 1];
+    for (int item = threadIdx.x; item < NK * TY; item += G::THREADS) {
+      const int kz = item / TY, yl = item % TY;
+      const V zk = s_Z[kz * (TY + 1) + yl], zm = s_Z[((N - kz) % N) * (TY + 1) + yl];
+      const int64_t at = ((int64_t)kz * N + x) * N + y0 + yl;
+      A[at] = cmake<V>((T)0.5 * (zk.x + zm.x), (T)0.5 * (zk.y - zm.y));
+      B[at] = cmake<V>((T)0.5 * (zk.y + zm.y), (T)-0.5 * (zk.x - zm.x));
+    }
+  }
+}
+
+template <typename T, int N>
+void launch_adj_products_z(const T* lam, const T* D, const double* dsum, T* const* H5, vec2_t<T>* const* out6,
+                           const vec2_t<T>* tw, cudaStream_t s) {
+  using G = AZGeom<T, N>;
+  AdjZArgs<T> a;
+  a.lam = lam; a.D = D; a.dsum = dsum;
+  for (int i = 0; i < 5; ++i) a.h[i] = H5[i];
+  for (int i = 0; i < 6; ++i) a.out[i] = out6[i];
+  raise_smem_limit<k_adj_products_z<T, N>>(G::SMEM);
+  k_adj_products_z<T, N><<<dim3(N / G::TY, N), G::THREADS, G::SMEM, s>>>(a, tw);
+}
+
 #define DGP_INST_Z(T, N)                                                                          \
   template void launch_fft_z_r2c<T, N>(const T*, int64_t, vec2_t<T>*, int64_t, int, ZPrologue,     \
                                        const vec2_t<T>*, cudaStream_t);                            \
-  template void launch_fft_z_c2r<T, N>(const FieldSet<T>&, T* const*, int, const vec2_t<T>*, cudaStream_t);
+  template void launch_fft_z_c2r<T, N>(const FieldSet<T>&, T* const*, int, const vec2_t<T>*, cudaStream_t); \
+  template void launch_adj_products_z<T, N>(const T*, const T*, const double*, T* const*, vec2_t<T>* const*,   \
+                                            const vec2_t<T>*, cudaStream_t);
 #define DGP_INST_ZB(N)                                                                                  \
   template void launch_fft_z_r2c_batch<float, N>(const float* const*, float2* const*, const ZPrologue*, int,  \
                                                  const float2*, cudaStream_t);                               \

@@ -124,9 +124,9 @@ void launch_fft_x_op(int op, const vec2_t<T>* in0, const vec2_t<T>* in1, const F
 //    phi = A delta + B D is Eq. FullDGP1.
 //  XOP_ZEL_ADJ: inputs (mask bits 1..3) Psibar_x, Psibar_y, Psibar_z; out0 =
 //    -(1/k^2) sum_j i k_j Psibar_j, the transpose of the Zel'dovich multiplier.
-//  XOP_ADJ_COMBINE: inputs P_xx, P_yy, P_zz, P_xy, P_xz, P_yz (spectra of
-//    H_ij(D) lam) and lam; out0 = -2 sum_ij h_ij P_ij + c2 (-1/kbar) lam over all
-//    nine i, j (off-diagonals twice), h_ij the Hessian multipliers.
+//  XOP_ADJ_COMBINE: inputs P_yy - P_xx, P_zz - P_xx, P_xy, P_xz, P_yz (P_ij the spectra of
+//    H_ij(D) lam) and lam; out0 = -2 sum_ij h_ij P_ij + 2 P_xx + c2 (-1/kbar) lam over all
+//    nine i, j (off-diagonals twice), h_ij the Hessian multipliers (h_xx = 1 - h_yy - h_zz).
 template <typename T, int N>
 void launch_fft_x_adj(int op, const FieldSet<T>& in, int in_mask, const FieldSet<T>& out, const KParams& kp,
                       const vec2_t<T>* tw, cudaStream_t s);
@@ -258,19 +258,23 @@ template <typename T>
 void launch_sph_update(const T* S, T* D, int64_t m, double alpha, double* partials, int nblocks, cudaStream_t s);
 
 // Adjoint relaxation (J^T lam = g on mean-free fields, w-split as the forward
-// iteration).  d = D - mean(D) (mean = dsum / m), diag = 2 (1 - w) d + alpha.
-//  products: P[f m + i] = H_f lam for f = xx (= d - yy - zz), yy, zz, xy, xz, yz, H5 = yy, zz, xy, xz, yz.
-//  update_a: u = (g - 2 w d lam - Q) / diag; partials[b][2] = (sum u, sum diag (lam - u)).
+// iteration).  d = D - mean(D) (mean = dsum / m), diag = 2 (1 - w) d + alpha.  With h_xx = 1 - h_yy - h_zz
+// the sum over all h_ij F[H_ij lam] is F[H_xx lam] + h_yy F[(H_yy - H_xx) lam] + h_zz F[(H_zz - H_xx) lam] + the
+// off-diagonals: the first term needs no transform (its mean is absorbed by the constant c below).
+//  products_z: the z half spectra of (H_yy - H_xx) lam, (H_zz - H_xx) lam, H_xy lam, H_xz lam, H_yz lam, lam
+//    (H5 = yy, zz, xy, xz, yz).
+//  update_a: u = (g - 2 w d lam - Q + 2 H_xx lam) / diag, Q the transformed terms (null: lam = 0, u = g / diag);
+//    partials[b][2] = (sum u, sum diag (lam - u)).
 //  update_b: sums = [sum u, sum diag (lam - u), sum 1/diag]; lam <- u + c / diag with
 //    c = -mean(u) / mean(1/diag) (lam stays mean-free); partials[b] = sum |diag (lam_old - u)
 //    - mean| (the projected residual of the previous lam).
 //  inv_diag: partials[b][2] = (sum 1/diag, number of points with diag <= 0).
+template <typename T, int N>
+void launch_adj_products_z(const T* lam, const T* D, const double* dsum, T* const* H5, vec2_t<T>* const* out6,
+                           const vec2_t<T>* tw, cudaStream_t s);
 template <typename T>
-void launch_adj_products(const T* lam, const T* D, const double* dsum, T* const* H5, T* P, int64_t m,
-                         cudaStream_t s);
-template <typename T>
-void launch_adj_update_a(const T* lam, const T* D, const double* dsum, const T* g, const T* Q, T* u, int64_t m,
-                         double alpha, double w, double* partials, int nblocks, cudaStream_t s);
+void launch_adj_update_a(const T* lam, const T* D, const double* dsum, const T* g, const T* Q, T* const* H5, T* u,
+                         int64_t m, double alpha, double w, double* partials, int nblocks, cudaStream_t s);
 template <typename T>
 void launch_adj_update_b(T* lam, const T* D, const double* dsum, const T* u, int64_t m, double alpha, double w,
                          const double* sums, double* partials, int nblocks, cudaStream_t s);

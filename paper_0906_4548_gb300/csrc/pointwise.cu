@@ -443,40 +443,47 @@ __device__ __forceinline__ T block_mean_d(const double* dsum, int64_t m) {
   return s_mean;
 }
 
-template <typename T>
-__global__ void __launch_bounds__(256) k_adj_products(const T* __restrict__ lam, const T* __restrict__ D,
-                                                      const double* __restrict__ dsum, const T* __restrict__ hyy,
-                                                      const T* __restrict__ hzz, const T* __restrict__ hxy,
-                                                      const T* __restrict__ hxz, const T* __restrict__ hyz,
-                                                      T* __restrict__ P, int64_t m) {
-  const T mean = block_mean_d<T>(dsum, m);
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-    const T l = lam[i], a = hyy[i], b = hzz[i];
-    P[i] = ((D[i] - mean) - a - b) * l;
-    P[m + i] = a * l;
-    P[2 * m + i] = b * l;
-    P[3 * m + i] = hxy[i] * l;
-    P[4 * m + i] = hxz[i] * l;
-    P[5 * m + i] = hyz[i] * l;
+// A thread's sums: float pairs for FP32 data (FP64 additions of converted values bound these passes
+// to the FP64 pipe), FP64 otherwise.
+template <typename T> struct ThreadSum {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double v) { s += v; }
+  __device__ __forceinline__ void add_inverse(double v) { s += 1.0 / v; }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <> struct ThreadSum<float> {
+  FP s{0.f, 0.f};
+  __device__ __forceinline__ void add(float v) { fp_acc(s, FP{v, 0.f}); }
+  __device__ __forceinline__ void add_inverse(float v) {  // 1 / v = r + r (1 - r v), the remainder exact
+    const float r = 1.f / v;
+    fp_acc(s, FP{r, r * fmaf(-r, v, 1.f)});
   }
-}
+  __device__ __forceinline__ double value() const { return (double)s.hi + (double)s.lo; }
+};
 
 template <typename T>
 __global__ void __launch_bounds__(256) k_adj_update_a(const T* __restrict__ lam, const T* __restrict__ D,
                                                       const double* __restrict__ dsum, const T* __restrict__ g,
-                                                      const T* __restrict__ Q, T* __restrict__ u, int64_t m,
+                                                      const T* __restrict__ Q, const T* __restrict__ hyy,
+                                                      const T* __restrict__ hzz, T* __restrict__ u, int64_t m,
                                                       T alpha, T w, double* __restrict__ partials) {
   const T mean = block_mean_d<T>(dsum, m);
-  double su = 0.0, sr = 0.0;
+  ThreadSum<T> su, sr;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-    const T d = D[i] - mean, l = lam[i];
+    const T d = D[i] - mean;
     const T diag = (T)2 * ((T)1 - w) * d + alpha;
-    const T ui = (g[i] - (T)2 * w * d * l - Q[i]) / diag;
+    T l = (T)0, rest = (T)0;
+    if (Q) {
+      l = lam[i];
+      const T xx = d - hyy[i] - hzz[i];
+      rest = (T)2 * (w * d - xx) * l + Q[i];
+    }
+    const T ui = (g[i] - rest) / diag;
     u[i] = ui;
-    su += (double)ui;
-    sr += (double)(diag * (l - ui));
+    su.add(ui);
+    sr.add(diag * (l - ui));
   }
-  double v[2] = {su, sr};
+  double v[2] = {su.value(), sr.value()};
   block_sum<2>(v);
   if (threadIdx.x == 0) {
     partials[2 * blockIdx.x] = v[0];
@@ -492,15 +499,15 @@ __global__ void __launch_bounds__(256) k_adj_update_b(T* __restrict__ lam, const
   const T mean = block_mean_d<T>(dsum, m);
   const T c = (T)(-(sums[0] / (double)m) / (sums[2] / (double)m));
   const T rmean = (T)(sums[1] / (double)m);
-  double sa = 0.0;
+  ThreadSum<T> sa;
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
     const T d = D[i] - mean;
     const T diag = (T)2 * ((T)1 - w) * d + alpha;
     const T ui = u[i];
-    sa += (double)fabs(diag * (lam[i] - ui) - rmean);
+    sa.add(fabs(diag * (lam[i] - ui) - rmean));
     lam[i] = ui + c / diag;
   }
-  double v[1] = {sa};
+  double v[1] = {sa.value()};
   block_sum<1>(v);
   if (threadIdx.x == 0) partials[blockIdx.x] = v[0];
 }
@@ -509,13 +516,14 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_adj_inv_diag(const T* __restrict__ D, const double* __restrict__ dsum,
                                                       int64_t m, T alpha, T w, double* __restrict__ partials) {
   const T mean = block_mean_d<T>(dsum, m);
-  double s = 0.0, nbad = 0.0;
+  ThreadSum<T> s;
+  float nbad = 0.f;  // at most a thread's share of the points
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
     const T diag = (T)2 * ((T)1 - w) * (D[i] - mean) + alpha;
-    if (diag > (T)0) s += 1.0 / (double)diag;
-    else nbad += 1.0;
+    if (diag > (T)0) s.add_inverse(diag);
+    else nbad += 1.f;
   }
-  double v[2] = {s, nbad};
+  double v[2] = {s.value(), (double)nbad};
   block_sum<2>(v);
   if (threadIdx.x == 0) {
     partials[2 * blockIdx.x] = v[0];
@@ -530,14 +538,9 @@ __global__ void k_axpy(const T* __restrict__ x, const T* __restrict__ y, T* __re
 }
 
 template <typename T>
-void launch_adj_products(const T* lam, const T* D, const double* dsum, T* const* H5, T* P, int64_t m,
-                         cudaStream_t s) {
-  k_adj_products<T><<<num_sms() * 4, 256, 0, s>>>(lam, D, dsum, H5[0], H5[1], H5[2], H5[3], H5[4], P, m);
-}
-template <typename T>
-void launch_adj_update_a(const T* lam, const T* D, const double* dsum, const T* g, const T* Q, T* u, int64_t m,
-                         double alpha, double w, double* partials, int nblocks, cudaStream_t s) {
-  k_adj_update_a<T><<<nblocks, 256, 0, s>>>(lam, D, dsum, g, Q, u, m, (T)alpha, (T)w, partials);
+void launch_adj_update_a(const T* lam, const T* D, const double* dsum, const T* g, const T* Q, T* const* H5, T* u,
+                         int64_t m, double alpha, double w, double* partials, int nblocks, cudaStream_t s) {
+  k_adj_update_a<T><<<nblocks, 256, 0, s>>>(lam, D, dsum, g, Q, H5[0], H5[1], u, m, (T)alpha, (T)w, partials);
 }
 template <typename T>
 void launch_adj_update_b(T* lam, const T* D, const double* dsum, const T* u, int64_t m, double alpha, double w,
@@ -555,9 +558,8 @@ void launch_axpy(const T* x, const T* y, T* out, int64_t m, cudaStream_t s) {
 }
 
 #define DGP_INST_PW(T)                                                                         \
-  template void launch_adj_products<T>(const T*, const T*, const double*, T* const*, T*, int64_t, cudaStream_t); \
-  template void launch_adj_update_a<T>(const T*, const T*, const double*, const T*, const T*, T*, int64_t,     \
-                                       double, double, double*, int, cudaStream_t);                           \
+  template void launch_adj_update_a<T>(const T*, const T*, const double*, const T*, const T*, T* const*, T*,   \
+                                       int64_t, double, double, double*, int, cudaStream_t);                  \
   template void launch_adj_update_b<T>(T*, const T*, const double*, const T*, int64_t, double, double,         \
                                        const double*, double*, int, cudaStream_t);                            \
   template void launch_adj_inv_diag<T>(const T*, const double*, int64_t, double, double, double*, int,         \
