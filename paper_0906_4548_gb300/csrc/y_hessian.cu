@@ -15,9 +15,10 @@
 //
 // Memory: reads three half spectra and writes six, in place: G0, G1 and N arrive in the buffers of
 // H_yz, H_xz and N, each the last output formed from it, and a CTA reads only the rows it writes.
-// Bound by memory: 9 half spectra (608 MB at 256^3) in 98 us, 0.91 of the copy rate.  The passes it
+// Bound by memory: 9 half spectra (608 MB at 256^3) in 93.5 us, 0.96 of the copy rate (part of what it
+// reads comes from L2).  The passes it
 // replaces (an x pass writing all six spectra, then six inverse y transforms in place) moved 19 half
-// spectra in 95 + 110 us; this one and the x pass move 13 in 98 + 80 us.
+// spectra in 95 + 110 us; this one and the x pass move 13 in 93.5 + 67.5 us.
 #include "fft_core.cuh"
 #include "kernels.cuh"
 
@@ -25,19 +26,20 @@ namespace dgp {
 
 template <typename T, int N> struct YHGeom {
   static constexpr int N1 = Split<N>::N1, N2 = Split<N>::N2;
-    // rows per CTA, all of one kz plane.  FP32 at 256^3 with 16, 8, 4 rows and 24 warps of 80
-  // registers per SM: 131, 119, 117 us; 16 warps of 128 registers: 116, 98, 99 us.  The extra registers let a thread's 16 loads and
-  // its transform overlap, which hides the latency better than more warps.
-  static constexpr int P = sizeof(T) == 4 ? 8 : 4;
+  // rows per CTA, all of one kz plane.  FP32 at 256^3 with 16, 8, 4 rows and 24 warps of 80 registers
+  // per SM: 131, 119, 117 us; 16 warps of 128 registers: 116, 98, 99 us.  The extra registers let a
+  // thread's 16 loads and its transform overlap, which hides the latency better than more warps.
+  // 512^3: 4 rows and five CTAs per SM (8 rows, two CTAs: 1061 us; 4 rows, four, five, six: 937, 898, 939).
+  static constexpr int P = sizeof(T) == 4 && N < 512 ? 8 : 4;
   static constexpr int THREADS = P * N1;
   // row stride of the transpose (complex), N2 mod 16 when N2 < N1 so that the packed first stage's
   // rows of a half-warp fall on different banks
   static constexpr int RS0 = N1 * (N2 + 1);
   static constexpr int RS = N2 < N1 ? RS0 + ((N2 - RS0 % 16) % 16 + 16) % 16 : RS0;
   static constexpr size_t SMEM = sizeof(vec2_t<T>) * (N + 2 * (size_t)P * RS);
-  static constexpr int MINB = sizeof(T) == 4 ? (N <= 256 ? 512 / THREADS : 2) : 1;
+  static constexpr int MINB = sizeof(T) == 4 ? (N <= 256 ? 512 / THREADS : 5) : 1;
   // keep the row of G0 (G1) in registers for the outputs formed from it; a 32-point first stage has
-  // no room for that and reads the row again (512^3: 1085 us against 1111 us with spills)
+  // no room for that and reads the row again
   static constexpr bool KEEP = N <= 256;
   // CTAs of one realisation, and whether an output group (those of G0, of G1, N) has CTAs of its own:
   // below two CTAs per SM the chain of six transforms in a CTA is what takes the time (64^3: 7.8 us
@@ -65,7 +67,9 @@ __global__ void __launch_bounds__(YHGeom<T, N>::THREADS, YHGeom<T, N>::MINB)
   for (int i = threadIdx.x; i < N; i += G::THREADS) s_tw[i] = g_tw[N + i];
   const int lane = threadIdx.x % N1, row = threadIdx.x / N1;
   constexpr int BPP = N / P;  // CTAs per kz plane
-  const int kz = blockIdx.x / BPP, x0 = (blockIdx.x % BPP) * P;
+  // planes from the last to the first: those the x pass wrote last are still in L2 (256^3: 98 -> 93.5 us)
+  const int blk = gridDim.x - 1 - blockIdx.x;
+  const int kz = blk / BPP, x0 = (blk % BPP) * P;
   const int64_t plane = (int64_t)kz * N * N;
   // stage one: P x N2 tasks (a row and its column c1) on the first threads
   const int r1 = threadIdx.x / N2, c1 = threadIdx.x % N2;
