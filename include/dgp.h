@@ -330,10 +330,10 @@ int dgp_set_tile_config(dgp_ctx *c, int y_threads);
  * data at n = 128 or 256, when the device co-schedules a thread-block cluster
  * of n / 16 CTAs, an iteration forms the six spectra and transforms them back
  * along x and y in one launch (a cluster per kz plane exchanging through
- * distributed shared memory) instead of an x pass and a six-field y pass; the
- * six spectra then cross memory once instead of three times.  The results
+ * distributed shared memory) instead of an x pass and a y pass; the three
+ * spectra between those two then never cross memory.  The results
  * are the same up to rounding order.  On a GB300 at 256^3 the fused launch
- * took 352 us against 240 us for the two passes it replaces, so it is off by
+ * took 352 us against 161 us for the two passes it replaces, so it is off by
  * default.  dgp_set_hessian_fusion turns it on (on != 0) or off (0, the
  * default); dgp_hessian_fusion sets *active to 1 when the context's solves
  * use it.  DGP_E_INVALID for a NULL argument. */

@@ -735,7 +735,7 @@ __global__ void __launch_bounds__(XGeom<T, N>::THREADS, XGeom<T, N>::MIN_BLOCKS)
 }
 
 // ---------------------------------------------------------------------------
-// Hessian x pass for FP32 data with the spectrum in shared memory (N <= 256).
+// Hessian x pass for FP32 data.
 //
 // The same work as k_fft_x's Hessian operation for one kz plane and TY ky columns, with the
 // x transforms as four-step stages through a [x][ky] tile in shared memory: the forward transform
@@ -743,7 +743,9 @@ __global__ void __launch_bounds__(XGeom<T, N>::THREADS, XGeom<T, N>::MIN_BLOCKS)
 // output's inverse starts from that order, forming the multiplier as it reads.
 template <int N> struct XSGeom {
   static constexpr int N1 = Split<N>::N1, N2 = Split<N>::N2;
-  static constexpr int TY = 16;
+  // 512^3: 8 columns, so that two CTAs of 128 registers fit (the pass with the spectrum of 16 columns in
+  // the registers of one CTA of 512 threads took 702 us against 647)
+  static constexpr int TY = N == 512 ? 8 : 16;
   static constexpr int THREADS = TY * N1;
   static constexpr int TILE = N * TY;  // complex
   static constexpr size_t SMEM = sizeof(float2) * ((size_t)N + 2 * (size_t)TILE);  // phase table, two tiles
@@ -751,8 +753,8 @@ template <int N> struct XSGeom {
   // 256^3) instead of being read from shared memory for every output; half the shared-memory
   // instructions, which are what the pass waits for: 75 -> 67.5 us.  At 128^3 the tile version in 64
   // registers lets all 520 CTAs run at once (15.9 us against 17.6 with REG, 17.8 with three per SM).
-  static constexpr bool REG = N != 128;
-  static constexpr int MINB = N == 128 ? 4 : THREADS < 128 ? 6 : 512 / THREADS;
+  static constexpr bool REG = N != 128 && N != 512;
+  static constexpr int MINB = N == 512 ? 2 : N == 128 ? 4 : THREADS < 128 ? 6 : 512 / THREADS;
 };
 
 template <int N, int RB>
@@ -874,7 +876,7 @@ static void launch_x(const XArgs<T>* a, int count, const vec2_t<T>* tw, cudaStre
                                                                           : sizeof(T) * 2 * Split<N>::N2 * G::THREADS);
   const size_t per_bin = PK ? sizeof(double) * 2 * NBS : 0;
   const size_t smem = base + tables + per_bin * a[0].nbins;
-  if constexpr (OP == XOP_HESSIAN && sizeof(T) == 4 && N <= 256) {
+  if constexpr (OP == XOP_HESSIAN && sizeof(T) == 4) {
     launch_xs<N, RB>(a, count, tw, s);  // the shared-memory version of the same pass
   } else {
     raise_smem_limit<k_fft_x<T, N, OP, RB>>(base + tables + per_bin * (N / 2));
@@ -968,14 +970,14 @@ void launch_fft_x_rc(const FieldSet<T>& in, int in_mask, const KParams& kp, cons
 // barrier each CTA takes TY x rows of the plane: it reads their N ky values from the CTAs of
 // the cluster (distributed shared memory, TY consecutive values from each), transforms them
 // back along y and writes the rows of the output in the layout (kz, x, y) that the relaxation
-// pass reads.  An iteration then needs no six-field inverse y pass: its 12 S of memory traffic
-// (read and write of six half spectra) are gone and the six outputs cross memory once.  Two
+// pass reads.  An iteration then needs no Hessian y pass: the three half spectra that the x pass
+// writes for it never cross memory.  Two
 // alternating exchange buffers let one cluster barrier per output order the writes of one
 // output after the reads of the output before it; a last barrier keeps every CTA resident
 // until the others have read its buffers.  Measured on a GB300 at 256^3 (clusters of 16):
-// 352 us per launch against 240 us for the x pass and six-field y pass it replaces.  The x
-// pass is latency-bound at 16 warps per SM and the y work adds to its time rather than
-// hiding in it, so the fused pass is opt-in (dgp_set_hessian_fusion).
+// 352 us per launch against 161 us for the x pass and the Hessian y pass (k_y_hessian) it
+// replaces.  The x pass is latency-bound at 16 warps per SM and the y work adds to its time
+// rather than hiding in it, so the fused pass is opt-in (dgp_set_hessian_fusion).
 template <int N> struct XYGeom {
   static constexpr int N1 = Split<N>::N1, N2 = Split<N>::N2;
   static constexpr int TY = 16;                  // ky columns per CTA; x rows per CTA in the y stage
