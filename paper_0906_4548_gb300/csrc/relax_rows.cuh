@@ -28,17 +28,22 @@ namespace dgp {
 // rounds of the 8 lanes, the second half empty, and D_new goes through shared memory to the lanes of
 // the forward transform.  (Four lanes of 24 samples need 128 registers and leave 8 warps per SM to a
 // single 96^3 mesh: 25 us against 22 for rows spread over the CTA.)
-template <int N> struct RowSplit {
+// WIDE: twice the lanes per row (96: the same), and after the second stage the values of a field pair
+// go through the row's slots to all of them, N1 to a lane.
+template <int N, bool WIDE> struct RowSplit {
   static constexpr int N1 = Split<N>::N1, N2 = Split<N>::N2;
   static constexpr bool PHASES = true;
 };
-template <> struct RowSplit<48> { static constexpr int N1 = 12, N2 = 4; static constexpr bool PHASES = false; };
-template <> struct RowSplit<96> { static constexpr int N1 = 12, N2 = 8; static constexpr bool PHASES = false; };
+template <> struct RowSplit<48, false> { static constexpr int N1 = 12, N2 = 4; static constexpr bool PHASES = false; };
+template <> struct RowSplit<96, false> { static constexpr int N1 = 12, N2 = 8; static constexpr bool PHASES = false; };
+template <> struct RowSplit<32, true> { static constexpr int N1 = 4, N2 = 8; static constexpr bool PHASES = false; };
+template <> struct RowSplit<48, true> { static constexpr int N1 = 6, N2 = 8; static constexpr bool PHASES = false; };
+template <> struct RowSplit<96, true> { static constexpr int N1 = 12, N2 = 8; static constexpr bool PHASES = false; };
 
-template <int N> struct RowGeom {
-  static constexpr int N1 = RowSplit<N>::N1, N2 = RowSplit<N>::N2, Q = (N1 + N2 - 1) / N2;
-  static constexpr bool EVEN = N1 % N2 == 0;  // every round of the second stage is full
-  static constexpr int PTS = Q * N2;          // values of a lane after it
+template <int N, bool WIDE> struct RowGeom {
+  static constexpr int N1 = RowSplit<N, WIDE>::N1, N2 = RowSplit<N, WIDE>::N2, Q = (N1 + N2 - 1) / N2;
+  static constexpr bool EVEN = WIDE || N1 % N2 == 0;  // a lane ends with the samples of its column
+  static constexpr int PTS = WIDE ? N1 : Q * N2;      // values of a lane after the inverse transform
   static constexpr int TY = 16, THREADS = TY * N2, WARPS = THREADS / 32;
   static constexpr int NK = N / 2 + 1;
   static constexpr int NBOX = (NK + 255) / 256;
@@ -102,21 +107,22 @@ __device__ __forceinline__ void rdft(const float (&x)[R], float2 (&X)[R / 2 + 1]
 }
 
 // W_N^{k1 c} of the four-step split from the table in shared memory
-template <int N> __device__ __forceinline__ float2 row_phase(const float2* s_tw, int k1, int c) {
-  if constexpr (RowSplit<N>::PHASES) return s_tw[k1 * RowSplit<N>::N2 + c];
+template <int N, bool WIDE> __device__ __forceinline__ float2 row_phase(const float2* s_tw, int k1, int c) {
+  if constexpr (RowSplit<N, WIDE>::PHASES) return s_tw[k1 * RowSplit<N, WIDE>::N2 + c];
   else return s_tw[k1 * c];
 }
 
 // the row's slots: those from N / 2 on are in the second tile
-template <int N> using RowSlots = TileSlots<RowGeom<N>::N1, RowGeom<N>::N2, RowGeom<N>::FIELD - (N / 2) * 128>;
+template <int N, bool WIDE>
+using RowSlots = TileSlots<RowGeom<N, WIDE>::N1, RowGeom<N, WIDE>::N2, RowGeom<N, WIDE>::FIELD - (N / 2) * 128>;
 
 // Inverse z transform of the pair in buf: on return a[i], b[i] with i = q + Q k2 are the two fields at
-// z = k1 + N1 k2, k1 = c + N2 q (zero where k1 >= N1); z = c + N2 i when N1 is a multiple of N2.
-template <int N>
+// z = k1 + N1 k2, k1 = c + N2 q (zero where k1 >= N1); z = c + N2 i when EVEN.
+template <int N, bool WIDE>
 __device__ __forceinline__ void row_pair_inverse(unsigned char* buf, const float2* s_tw, int r, int c,
-                                                 float (&a)[RowGeom<N>::PTS], float (&b)[RowGeom<N>::PTS]) {
-  using G = RowGeom<N>;
-  using S = RowSlots<N>;
+                                                 float (&a)[RowGeom<N, WIDE>::PTS], float (&b)[RowGeom<N, WIDE>::PTS]) {
+  using G = RowGeom<N, WIDE>;
+  using S = RowSlots<N, WIDE>;
   constexpr int N1 = G::N1, N2 = G::N2, Q = G::Q;
   {
     float2 v[N1];
@@ -145,9 +151,36 @@ __device__ __forceinline__ void row_pair_inverse(unsigned char* buf, const float
     dft_regs<N1, N / N1>(v, s_tw);
 #pragma unroll
     for (int k1 = 0; k1 < N1; ++k1)
-      tile_at(buf, S::by_col(off_d, k1)) = k1 == 0 ? v[k1] : cmul(v[k1], row_phase<N>(s_tw, k1, c));
+      tile_at(buf, S::by_col(off_d, k1)) = k1 == 0 ? v[k1] : cmul(v[k1], row_phase<N, WIDE>(s_tw, k1, c));
   }
   __syncwarp();
+  if constexpr (WIDE) {
+    // rows k1 on the lanes that have one; then sample z to the slot of line z, and lane c takes its column
+    float2 u[Q][N2];
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      if (c + N2 * q >= N1) continue;
+      const int base = S::by_row_base(c + N2 * q, r);
+#pragma unroll
+      for (int j2 = 0; j2 < N2; ++j2) u[q][j2] = tile_at(buf, S::by_row(base, j2));
+      dft_regs<N2, N / N2>(u[q], s_tw);
+    }
+    __syncwarp();
+#pragma unroll
+    for (int q = 0; q < Q; ++q) {
+      if (c + N2 * q >= N1) continue;
+#pragma unroll
+      for (int k2 = 0; k2 < N2; ++k2) tile_at(buf, S::folded(c + N2 * q + N1 * k2, r)) = u[q][k2];
+    }
+    __syncwarp();
+#pragma unroll
+    for (int i = 0; i < N1; ++i) {
+      const float2 v = tile_at(buf, S::folded(c + N2 * i, r));
+      a[i] = v.x;
+      b[i] = -v.y;
+    }
+    return;
+  }
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
     if (!G::EVEN && c + N2 * q >= N1) {
@@ -170,11 +203,11 @@ __device__ __forceinline__ void row_pair_inverse(unsigned char* buf, const float
 
 // Forward z transform of the row whose values at z = c + N2 j1 are d[j1]; the half spectrum goes to
 // the first tile of buf in the tile layout (line kz, row r).
-template <int N>
+template <int N, bool WIDE>
 __device__ __forceinline__ void row_forward(unsigned char* buf, const float2* s_tw, int r, int c,
-                                            const float (&d)[RowGeom<N>::N1]) {
-  using G = RowGeom<N>;
-  using S = RowSlots<N>;
+                                            const float (&d)[RowGeom<N, WIDE>::N1]) {
+  using G = RowGeom<N, WIDE>;
+  using S = RowSlots<N, WIDE>;
   constexpr int N1 = G::N1, N2 = G::N2;
   {
     float2 V[N1 / 2 + 1];
@@ -182,7 +215,7 @@ __device__ __forceinline__ void row_forward(unsigned char* buf, const float2* s_
     const int base = S::line(c, r);
 #pragma unroll
     for (int k1 = 0; k1 <= N1 / 2; ++k1) {
-      const float2 w = row_phase<N>(s_tw, k1, c);
+      const float2 w = row_phase<N, WIDE>(s_tw, k1, c);
       const float2 t = k1 == 0 ? V[0] : k1 == N1 / 2 ? make_float2(V[k1].x * w.x, V[k1].x * w.y) : cmul(V[k1], w);
       tile_at(buf, S::by_col(base, k1)) = t;
     }
@@ -220,12 +253,25 @@ __device__ __forceinline__ void row_forward(unsigned char* buf, const float2* s_
   }
 }
 
+// Whether a pass takes the wide rows: FP64 arithmetic always (it is what the pass waits for: an FP64
+// instruction holds a quarter of the SM for some 60 cycles, at 32^3 and 48^3 there are too few warps for
+// 8 and 12 points a lane, at 96^3 a third of the lanes would idle; per solve of 23-26 evaluations 837 ->
+// 728, 1094 -> 904 and 3043 -> 2535 us), float pairs and any arithmetic at 48^3 where one mesh does not
+// fill the chip (float pairs at 32, 48, 96: 681 -> 636, 844 -> 759, 1333 -> 1284 us; FP32 at 48^3 766 ->
+// 737).  FP32 at 32^3 gains nothing, at 96^3 it loses (1154 -> 1236: the trip through the slots).
+template <int N, class AR, int RB> struct RowWide {
+  static constexpr bool F64 = std::is_same<typename AR::Sum, double>::value;
+  static constexpr bool EFT = std::is_same<AR, RxEFT>::value;
+  static constexpr bool W = (N == 32 || N == 48 || N == 96) && (F64 || (RB == 1 && (EFT || N == 48)));
+};
+
 template <int N, class AR, int RB>
-__global__ void __launch_bounds__(RowGeom<N>::THREADS, RowGeom<N>::MINB)
+__global__ void __launch_bounds__(RowGeom<N, RowWide<N, AR, RB>::W>::THREADS, RowGeom<N, RowWide<N, AR, RB>::W>::MINB)
     k_relax_rows(const __grid_constant__ RelaxTmaBatch<RB> batch, const float2* __restrict__ g_tw) {
   const RelaxTmaArgs& args = batch.a[RB > 1 ? blockIdx.z : 0];  // realisation of this CTA
   if (args.skip && *args.skip) return;
-  using G = RowGeom<N>;
+  constexpr bool WIDE = RowWide<N, AR, RB>::W;
+  using G = RowGeom<N, WIDE>;
   using Acc = typename AR::Acc;
   using Sum = typename AR::Sum;
   constexpr int N1 = G::N1, N2 = G::N2, TY = G::TY, ROWP = G::ROWP, WARPS = G::WARPS;
@@ -265,7 +311,7 @@ __global__ void __launch_bounds__(RowGeom<N>::THREADS, RowGeom<N>::MINB)
     mp[1] = (float)(m - (double)mp[0]);
     s_cnt[0] = s_cnt[1] = s_cnt[2] = s_cnt[3] = 0;
   }
-  for (int i = tid; i < N; i += G::THREADS) s_tw[i] = g_tw[(RowSplit<N>::PHASES ? N : 0) + i];
+  for (int i = tid; i < N; i += G::THREADS) s_tw[i] = g_tw[(RowSplit<N, WIDE>::PHASES ? N : 0) + i];
   __syncthreads();
   const double mean = s_mean[0];
   const float m_hi = reinterpret_cast<const float*>(s_mean + 1)[0];
@@ -300,12 +346,12 @@ __global__ void __launch_bounds__(RowGeom<N>::THREADS, RowGeom<N>::MINB)
   Acc acc[PTS];
   float ra[PTS], rb[PTS];
   wait(&bars[0], 0);
-  row_pair_inverse<N>(buf0, s_tw, r, c, ra, rb);
+  row_pair_inverse<N, WIDE>(buf0, s_tw, r, c, ra, rb);
 #pragma unroll
   for (int i = 0; i < PTS; ++i) AR::pair_a(acc[i], ra[i], rb[i]);
   if (last_warp(0) && wl == 0 && !gave_up()) issue(buf0, 0, 1, &bars[0]);  // pair C, the diagonal
   wait(&bars[1], 0);
-  row_pair_inverse<N>(buf1, s_tw, r, c, ra, rb);
+  row_pair_inverse<N, WIDE>(buf1, s_tw, r, c, ra, rb);
 #pragma unroll
   for (int i = 0; i < PTS; ++i) AR::pair_b(acc[i], ra[i], rb[i], rp);
   float* sD = reinterpret_cast<float*>(buf1);
@@ -318,7 +364,7 @@ __global__ void __launch_bounds__(RowGeom<N>::THREADS, RowGeom<N>::MINB)
     bulk_load((wl < TY ? sD : sS) + (wl % TY) * ROWP, src, N * 4, &bars[1]);
   }
   wait(&bars[0], 1);
-  row_pair_inverse<N>(buf0, s_tw, r, c, ra, rb);  // a, b: two diagonal second derivatives
+  row_pair_inverse<N, WIDE>(buf0, s_tw, r, c, ra, rb);  // a, b: two diagonal second derivatives
   wait(&bars[1], 1);
   Sum rsum{};
   FP acc_d{0.f, 0.f};  // sum of D_new: its mean is removed next iteration
@@ -353,12 +399,12 @@ __global__ void __launch_bounds__(RowGeom<N>::THREADS, RowGeom<N>::MINB)
   }
   __syncwarp();  // the row's slots of buf0 are read, its D_new is written
   if constexpr (G::EVEN) {
-    row_forward<N>(buf0, s_tw, r, c, ra);
+    row_forward<N, WIDE>(buf0, s_tw, r, c, ra);
   } else {
     float d[N1];
 #pragma unroll
     for (int j1 = 0; j1 < N1; ++j1) d[j1] = sD[r * ROWP + N2 * j1 + c];
-    row_forward<N>(buf0, s_tw, r, c, d);
+    row_forward<N, WIDE>(buf0, s_tw, r, c, d);
   }
   // ---- statistics: within a warp float pairs (FP64 for the FP64 policy), across warps FP64
   if constexpr (std::is_same<Sum, double>::value) {

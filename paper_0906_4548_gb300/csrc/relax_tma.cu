@@ -235,7 +235,7 @@ static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 
 template <int N>
 int relax_maps(float2* const* spec6, float2* const* snew2, RelaxMaps* out) {
-  using G = RowGeom<N>;
+  using G = RowGeom<N, false>;  // boxes and tiles are the same for wide rows
   const PFN_cuTensorMapEncodeTiled_v12000 enc = tensor_map_encoder();
   if (!enc) return 1;
   // the half spectrum S[kz][x][y] as floats: dim 0 = 2N floats along y, dim 1 = x, dim 2 = kz
@@ -261,13 +261,13 @@ void relax_set_maps(const RelaxMaps& maps, float2* Snew, RelaxTmaArgs* a) {
   a->Snew = Snew;
 }
 
-template <int N> int relax_tma_blocks() { return (N / RowGeom<N>::TY) * N; }
+template <int N> int relax_tma_blocks() { return (N / RowGeom<N, false>::TY) * N; }
 
 template <int N, class AR, int RB>
 static void launch_rt(const RelaxTmaArgs* a, int count, const float2* tw, cudaStream_t s) {
   RelaxTmaBatch<RB> b;
   for (int r = 0; r < count; ++r) b.a[r] = a[r];
-  using G = RowGeom<N>;
+  using G = RowGeom<N, RowWide<N, AR, RB>::W>;
   raise_smem_limit<k_relax_rows<N, AR, RB>>(G::SMEM);
   k_relax_rows<N, AR, RB><<<dim3(N / G::TY, N, count), G::THREADS, G::SMEM, s>>>(b, tw);
 }

@@ -24,6 +24,8 @@ template <int N1, int N2, int FOLD> struct TileSlots {
   static __host__ __device__ constexpr int odd4(int k1) { return N2 == 4 ? (k1 & 1) << 6 : 0; }
   // byte offset of line l, pencil r (first tile)
   static __device__ __forceinline__ int line(int l, int r) { return l * 128 + ((r * 8) ^ ((l & 7) << 4)); }
+  // line l of the N lines across both tiles, pencil r
+  static __device__ __forceinline__ int folded(int l, int r) { return line(l, r) + (l >= N1 * N2 / 2 ? FOLD : 0); }
   // sample N2 j1 + c, given line(c, r)
   static __device__ __forceinline__ int sample(int base, int j1) {
     return (base + j1 * N2 * 128) ^ (N2 == 4 ? (j1 & 1) << 6 : 0);
