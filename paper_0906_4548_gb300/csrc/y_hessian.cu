@@ -30,22 +30,27 @@ template <typename T, int N> struct YHGeom {
   // per SM: 131, 119, 117 us; 16 warps of 128 registers: 116, 98, 99 us.  The extra registers let a
   // thread's 16 loads and its transform overlap, which hides the latency better than more warps.
   // 512^3: 4 rows and five CTAs per SM (8 rows, two CTAs: 1061 us; 4 rows, four, five, six: 937, 898, 939).
-  static constexpr int P = sizeof(T) == 4 && N < 512 ? 8 : 4;
+  // FP64 at 32^3 and 48^3: 8 rows, since 4 leave half and more of a warp's lanes idle in stage one
+  // (4 x 4 and 4 x 3 tasks; a 32^3 solve 2973 -> 2874 us, 48^3 7832 -> 7297).
+  static constexpr int P = (sizeof(T) == 4 ? N < 512 : N == 32 || N == 48) ? 8 : 4;
   static constexpr int THREADS = P * N1;
   // row stride of the transpose (complex), N2 mod 16 when N2 < N1 so that the packed first stage's
   // rows of a half-warp fall on different banks
   static constexpr int RS0 = N1 * (N2 + 1);
   static constexpr int RS = N2 < N1 ? RS0 + ((N2 - RS0 % 16) % 16 + 16) % 16 : RS0;
-  static constexpr size_t SMEM = sizeof(vec2_t<T>) * (N + 2 * (size_t)P * RS);
-  static constexpr int MINB = sizeof(T) == 4 ? (N <= 256 ? 512 / THREADS : 5) : 1;
   // keep the row of G0 (G1) in registers for the outputs formed from it; a 32-point first stage has
   // no room for that and reads the row again
   static constexpr bool KEEP = N <= 256;
-  // CTAs of one realisation, and whether an output group (those of G0, of G1, N) has CTAs of its own:
-  // below two CTAs per SM the chain of six transforms in a CTA is what takes the time (64^3: 7.8 us
-  // against 9.3, 48^3: 7.8 against 10.9; at 96^3, four CTAs per SM, splitting is slower, 14.0 against 13.2)
+  // CTAs of one realisation.  Below two CTAs per SM the chain of six transforms in a CTA is what takes
+  // the time, so each output has threads of its own, three outputs in a CTA: those of G0 (whose buffer
+  // the third overwrites), and those of G1 with N.  FP64 solves against one CTA for all outputs of a
+  // field: 16^3 1750 -> 1592 us, 32^3 3221 -> 2973; FP32 the same within 1 %.  (At 96^3, four CTAs per SM, splitting by the field
+  // read was slower, 14.0 against 13.2 us.)
   static constexpr int CTAS = (N / 2 + 1) * (N / P);
   static constexpr bool SPLIT = CTAS <= 304;
+  static constexpr int OUTS = SPLIT ? 3 : 1;
+  static constexpr size_t SMEM = sizeof(vec2_t<T>) * (N + (SPLIT ? 3 : 2) * (size_t)P * RS);
+  static constexpr int MINB = sizeof(T) == 8 ? 1 : N == 512 ? 5 : SPLIT ? 1 : 512 / THREADS;
   static_assert(N % P == 0, "a CTA's rows share kz");
 };
 
@@ -54,7 +59,7 @@ template <typename T, int RB> struct YHBatch {
 };
 
 template <typename T, int N, int RB>
-__global__ void __launch_bounds__(YHGeom<T, N>::THREADS, YHGeom<T, N>::MINB)
+__global__ void __launch_bounds__(YHGeom<T, N>::THREADS * YHGeom<T, N>::OUTS, YHGeom<T, N>::MINB)
     k_y_hessian(const __grid_constant__ YHBatch<T, RB> yb, const vec2_t<T>* __restrict__ g_tw) {
   const YHessArgs<T>& args = yb.a[RB > 1 ? blockIdx.z : 0];
   if (args.skip && *args.skip) return;
@@ -63,8 +68,8 @@ __global__ void __launch_bounds__(YHGeom<T, N>::THREADS, YHGeom<T, N>::MINB)
   constexpr int N1 = G::N1, N2 = G::N2, P = G::P;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   V* s_tw = reinterpret_cast<V*>(smem_raw);  // the phase table
-  V* s_T = s_tw + N;                         // two transposes, alternating
-  for (int i = threadIdx.x; i < N; i += G::THREADS) s_tw[i] = g_tw[N + i];
+  V* s_T = s_tw + N;                         // two transposes, alternating (SPLIT: one per output)
+  for (int i = threadIdx.y * G::THREADS + threadIdx.x; i < N; i += G::THREADS * G::OUTS) s_tw[i] = g_tw[N + i];
   const int lane = threadIdx.x % N1, row = threadIdx.x / N1;
   constexpr int BPP = N / P;  // CTAs per kz plane
   // planes from the last to the first: those the x pass wrote last are still in L2 (256^3: 98 -> 93.5 us)
@@ -84,14 +89,14 @@ __global__ void __launch_bounds__(YHGeom<T, N>::THREADS, YHGeom<T, N>::MINB)
   V g[N1];
   __syncthreads();
   // outputs in the order H_yy, H_zz, H_yz (of G0), H_xy, H_xz (of G1), N
-  const int o0 = !G::SPLIT || blockIdx.y == 0 ? 0 : blockIdx.y == 1 ? 3 : 5;
-  const int o1 = !G::SPLIT || blockIdx.y == 2 ? 6 : blockIdx.y == 0 ? 3 : 5;
+  const int o0 = G::SPLIT ? 3 * blockIdx.y + threadIdx.y : 0;
+  const int o1 = G::SPLIT ? o0 + 1 : 6;
 #pragma unroll 1
   for (int o = o0; o < o1; ++o) {
     const int slot = o == 0 ? 0 : o == 1 ? 1 : o == 2 ? 4 : o == 3 ? 2 : o == 4 ? 3 : 5;
-    V* T1 = s_T + (o & 1) * (P * G::RS);
+    V* T1 = s_T + (G::SPLIT ? threadIdx.y : o & 1) * (P * G::RS);
     if (act1) {
-      if (!G::KEEP || o == 0 || o == 3 || o == 5 || (o == 4 && nyq_z)) {
+      if (!G::KEEP || G::SPLIT || o == 0 || o == 3 || o == 5 || (o == 4 && nyq_z)) {
         const V* src = o < 3 ? args.f[4] + row1 : o == 5 ? args.f[5] + row1 : (o == 4 && nyq_z) ? aux_z : args.f[3] + row1;
 #pragma unroll
         for (int j1 = 0; j1 < N1; ++j1) g[j1] = src[N2 * j1 + c1];
@@ -137,7 +142,7 @@ __global__ void __launch_bounds__(YHGeom<T, N>::THREADS, YHGeom<T, N>::MINB)
     }
     // With N1 == N2 a row's threads are the same in both stages and lie in one warp.  After this
     // point every thread that reads the rows this output overwrites has read them.
-    if constexpr (N1 == N2) __syncwarp();
+    if constexpr (N1 == N2 && !G::SPLIT) __syncwarp();
     else __syncthreads();
     V u[N2];
     const V* Tp = T1 + row * G::RS + lane * (N2 + 1);
@@ -156,7 +161,8 @@ static void launch_yh(const YHessArgs<T>* a, int count, const vec2_t<T>* tw, cud
   raise_smem_limit<k_y_hessian<T, N, RB>>(G::SMEM);
   YHBatch<T, RB> yb;
   for (int r = 0; r < count; ++r) yb.a[r] = a[r];
-  k_y_hessian<T, N, RB><<<dim3((N / 2 + 1) * (N / G::P), G::SPLIT ? 3 : 1, count), G::THREADS, G::SMEM, s>>>(yb, tw);
+  k_y_hessian<T, N, RB><<<dim3((N / 2 + 1) * (N / G::P), G::SPLIT ? 2 : 1, count),
+                          dim3(G::THREADS, G::OUTS), G::SMEM, s>>>(yb, tw);
 }
 
 template <typename T, int N>
