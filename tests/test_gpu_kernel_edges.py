@@ -1,6 +1,6 @@
 """Edges of the estimator, sort, initial-condition and adjoint kernels: magnitudes far from one,
 shell counts and angle counts that do not fill a launch, pointers that are not 16-byte aligned, and
-every row split of the adjoint's fused z pass.
+every row split of the relaxation pass and of the adjoint's fused z pass.
 
 Tolerances: scaling a field by a power of two is exact in every step, so spectra scale exactly;
 a shorter list of shells and angles taken one at a time use the same sums, so they are equal; an
@@ -141,3 +141,25 @@ def test_fp32_adjoint_follows_fp64(dgp, torch_dev, n):
         finally:
             dgp.dgp_destroy(ctx)
     assert rel_l2(out["DGP_FP32"], out["DGP_FP64"]) < 1e-4
+
+
+@pytest.mark.parametrize("prec", ["DGP_FP32", "DGP_MIXED", "DGP_MIXED_EFT", "DGP_MIXED_F32R"])
+@pytest.mark.parametrize("n", [16, 32, 48, 64, 96])
+def test_relaxation_row_splits_follow_fp64(dgp, torch_dev, n, prec):
+    """Every row split of the relaxation pass in every arithmetic: forces of FP32-data solves to 1e-6
+    against an FP64 solve to 1e-12; the bound of the FP32-data paths, 1e-5."""
+    torch, dev = torch_dev
+    delta = torch.exp(_field(torch, dev, n, 21).double() * 0.25)
+    delta = (delta / delta.mean() - 1.0).float().double()
+    out = []
+    for p, tol, td in (("DGP_FP64", 1e-12, torch.float64), (prec, 1e-6, torch.float32)):
+        ctx = dgp.dgp_init(100.0 * n / 64, n, 1.0, OM, precision=getattr(dgp, p), tol=tol, max_iter=200)
+        try:
+            g = [torch.empty((n, n, n), dtype=td, device=dev) for _ in range(4)]  # phi and the forces
+            st, _ = dgp.dgp_solve_forces(ctx, 0.6, delta.to(td), *g, tol)
+            assert st == dgp.DGP_OK
+            torch.cuda.synchronize()
+            out.append(torch.stack(g[1:]).double().cpu().numpy())
+        finally:
+            dgp.dgp_destroy(ctx)
+    assert rel_l2(out[1], out[0]) < 1e-5
