@@ -57,9 +57,10 @@ SORT_EVERY = 8
 # SHA-256 of the sources the captured kernel was built from: when they have
 # changed since, the traffic is reported as null.
 NCU_TRAFFIC = {
-    "relax": {"bytes": 652.6e6, "sources": ['relax_tma.cu', 'tma.cuh', 'eft.cuh', 'fft_core.cuh', 'kernels.cuh', 'common.cuh'],
-              "sha256": "10664cba0c3d40605d047d2a008a8b42e05d6ce3eb56a750e3edaab2f3750327",
-              "profile": "profiles/k_relax_tma_256cube.md"},
+    "relax": {"bytes": 652.1e6, "sources": ['relax_tma.cu', 'relax_rows.cuh', 'tile_slots.cuh', 'tma.cuh', 'eft.cuh',
+                                            'fft_core.cuh', 'kernels.cuh', 'common.cuh'],
+              "sha256": "ef42b7c80c01cd6cd38e9c1d88167712ec3d70684b5966c5fc0e5aaee7bf2499",
+              "profile": "profiles/k_relax_rows_256cube.md"},
 }
 
 
