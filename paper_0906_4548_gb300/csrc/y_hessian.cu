@@ -44,8 +44,8 @@ template <typename T, int N> struct YHGeom {
   // CTAs of one realisation.  Below two CTAs per SM the chain of six transforms in a CTA is what takes
   // the time, so each output has threads of its own, three outputs in a CTA: those of G0 (whose buffer
   // the third overwrites), and those of G1 with N.  FP64 solves against one CTA for all outputs of a
-  // field: 16^3 1750 -> 1592 us, 32^3 3221 -> 2973; FP32 the same within 1 %.  (At 96^3, four CTAs per SM, splitting by the field
-  // read was slower, 14.0 against 13.2 us.)
+  // field: 16^3 1750 -> 1592 us, 32^3 3221 -> 2973; FP32 the same within 1 %.  (At 96^3, four CTAs
+  // per SM, splitting by the field read was slower, 14.0 against 13.2 us.)
   static constexpr int CTAS = (N / 2 + 1) * (N / P);
   static constexpr bool SPLIT = CTAS <= 304;
   static constexpr int OUTS = SPLIT ? 3 : 1;
