@@ -366,7 +366,8 @@ int dgp_set_blocking_sync(dgp_ctx *c, int on);
  * and gather for the whole class), its members iterate in lockstep, each
  * stopping by its own rules (members that have stopped skip at kernel entry),
  * and its relaxation iterations replay as one CUDA graph.  Every member ends
- * each step exactly as its own pm_step would leave it.  A realisation that
+ * each step as its own pm_step would leave it, up to the rounding of sums
+ * taken in another order.  A realisation that
  * forms no class is a context stepped alone on a stream of its own.  Each
  * class or lone context has one host worker thread, so classes run
  * concurrently; the contexts use blocking host waits.

@@ -974,8 +974,9 @@ class Engine : public EngineBase {
   // ---------------------------------------------------------------- classes of realisations
   // pm_step of every member of a class (same mesh, precision and stream; the nonlinear
   // mode), each kernel stage launched once for all members with the member on the grid's
-  // z (or y) index.  Every member ends in the state its own pm_step would leave it in:
-  // the same iterates, stop rules, warm start and reused end-of-step force.
+  // z (or y) index.  Every member ends in the state its own pm_step would leave it in, up to the
+  // rounding of sums taken in another order: the same iterates, stop rules, warm start and reused
+  // end-of-step force.
   cudaGraphExec_t class_exec = nullptr;  // the class's two-iteration graph (held by its first member)
 
   int step_class(EngineBase* const* members, int count, dgp_particles* parts, const double* a, const double* da,
@@ -1199,7 +1200,8 @@ class Engine : public EngineBase {
     launch_clear_verdicts(vb, n, st);
     int rc;
     if ((rc = check())) return rc;
-    // one iteration of the members in ks
+    // one iteration of the members in ks; a replay's relaxation takes the class's row split (n > 1), so that
+    // it gives the bits of the iterate it regenerates
     auto enqueue = [&](int it, bool control, const std::vector<int>& ks) {
       const int m = (int)ks.size();
       XReal<T> xr[kBatchMax];
@@ -1234,7 +1236,8 @@ class Engine : public EngineBase {
         PlaneArgs pa[kBatchMax];
         for (int i = 0; i < m; ++i) pa[i] = PlaneArgs{spec_in(ks[i], it), f6[i], kp[ks[i]], sk[i]};
         pf.run(KK_X_HESSIAN, 7.0 * m * SB, st, [&] { launch_plane_hessian_batch(N, pa, m, tw, st); });
-        pf.run(KK_RELAX, m * (7 * SB + 3 * RB), st, [&] { launch_relax_tma_batch<N>(e0->arith_mode(), ra, m, tw, st); });
+        pf.run(KK_RELAX, m * (7 * SB + 3 * RB), st,
+               [&] { launch_relax_tma_batch<N>(e0->arith_mode(), ra, m, n > 1, tw, st); });
         if (control) {
           pf.run(KK_REDUCE, 32.0 * m * e0->fblocks, st, [&] { launch_control_batch(yc, sk, m, st); });
         } else {
@@ -1259,7 +1262,8 @@ class Engine : public EngineBase {
         pf.run(KK_X_HESSIAN, 4.0 * m * SB, st, [&] { launch_fft_x_batch<T, N>(XOP_HESSIAN, xr, m, tw, st); });
         pf.run(KK_Y, 9.0 * m * SB, st, [&] { launch_y_hessian<T, N>(ya, m, tw, st); });
       }
-      pf.run(KK_RELAX, m * (7 * SB + 3 * RB), st, [&] { launch_relax_tma_batch<N>(e0->arith_mode(), ra, m, tw, st); });
+      pf.run(KK_RELAX, m * (7 * SB + 3 * RB), st,
+             [&] { launch_relax_tma_batch<N>(e0->arith_mode(), ra, m, n > 1, tw, st); });
       if (control) {
         pf.run(KK_Y, 2.0 * m * SB, st, [&] { launch_fft_y_batch<T, N>(f1, sk, yc, m, 1, false, tw, st, yt); });
       } else {

@@ -202,8 +202,11 @@ struct RelaxTmaArgs {
 template <int RB> struct RelaxTmaBatch {
   RelaxTmaArgs a[RB];
 };
+// of_class: the row split of a class's launches, else that of a single mesh (count = 1).  The two add in
+// different orders, so the replay of one member of a class says true as well.
 template <int N>
-void launch_relax_tma_batch(int arith, const RelaxTmaArgs* a, int count, const float2* tw, cudaStream_t s);
+void launch_relax_tma_batch(int arith, const RelaxTmaArgs* a, int count, bool of_class, const float2* tw,
+                            cudaStream_t s);
 
 // The Hessian passes of an iteration.  The x pass (XOP_HESSIAN) leaves three spectra in the buffers
 // of outputs 4, 3 and 5 (G0 = IFFT_x[D / k^2], G1 = IFFT_x[k_x D / k^2], N) and the auxiliary

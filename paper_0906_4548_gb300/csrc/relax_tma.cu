@@ -273,9 +273,9 @@ static void launch_rt(const RelaxTmaArgs* a, int count, const float2* tw, cudaSt
 }
 
 template <int N, class AR>
-static void launch_rt(const RelaxTmaArgs* a, int count, const float2* tw, cudaStream_t s) {
-  if (count == 1) launch_rt<N, AR, 1>(a, 1, tw, s);
-  else launch_rt<N, AR, kBatchMax>(a, count, tw, s);
+static void launch_rt(const RelaxTmaArgs* a, int count, bool of_class, const float2* tw, cudaStream_t s) {
+  if (of_class) launch_rt<N, AR, kBatchMax>(a, count, tw, s);
+  else launch_rt<N, AR, 1>(a, 1, tw, s);
 }
 
 template <int N>
@@ -286,16 +286,17 @@ void launch_relax_tma(int arith, const RelaxMaps& maps, const float* D, const do
   relax_set_maps(maps, Snew, &a);
   a.D = D; a.dsum = dsum; a.S = S; a.Dnew = Dnew; a.partials = partials; a.rp = rp;
   a.skip = skip; a.fault = fault; a.wait_ns = wait_ns; a.withhold = withhold;
-  launch_relax_tma_batch<N>(arith, &a, 1, tw, s);
+  launch_relax_tma_batch<N>(arith, &a, 1, false, tw, s);
 }
 
 template <int N>
-void launch_relax_tma_batch(int arith, const RelaxTmaArgs* a, int count, const float2* tw, cudaStream_t s) {
-  if (count < 1 || count > kBatchMax) return;
-  if (arith == ARITH_F64) launch_rt<N, RxF64>(a, count, tw, s);
-  else if (arith == ARITH_EFT) launch_rt<N, RxEFT>(a, count, tw, s);
-  else if (arith == ARITH_M32) launch_rt<N, RxM32>(a, count, tw, s);
-  else launch_rt<N, RxF32>(a, count, tw, s);
+void launch_relax_tma_batch(int arith, const RelaxTmaArgs* a, int count, bool of_class, const float2* tw,
+                            cudaStream_t s) {
+  if (count < 1 || count > (of_class ? kBatchMax : 1)) return;
+  if (arith == ARITH_F64) launch_rt<N, RxF64>(a, count, of_class, tw, s);
+  else if (arith == ARITH_EFT) launch_rt<N, RxEFT>(a, count, of_class, tw, s);
+  else if (arith == ARITH_M32) launch_rt<N, RxM32>(a, count, of_class, tw, s);
+  else launch_rt<N, RxF32>(a, count, of_class, tw, s);
 }
 
 #define DGP_INST_RT(N)                                                                                          \
@@ -304,7 +305,7 @@ void launch_relax_tma_batch(int arith, const RelaxTmaArgs* a, int count, const f
   template void launch_relax_tma<N>(int, const RelaxMaps&, const float*, const double*, const float*, float*,  \
                                     float2*, RelaxParams, double*, const float2*, cudaStream_t, const int*, int*, \
                                     unsigned long long, int);                                                 \
-  template void launch_relax_tma_batch<N>(int, const RelaxTmaArgs*, int, const float2*, cudaStream_t);
+  template void launch_relax_tma_batch<N>(int, const RelaxTmaArgs*, int, bool, const float2*, cudaStream_t);
 DGP_INST_RT(16)
 DGP_INST_RT(32)
 DGP_INST_RT(48)
