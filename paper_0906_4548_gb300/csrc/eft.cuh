@@ -31,6 +31,25 @@ __device__ __forceinline__ void fp_acc(FP& s, FP t) {
   s.hi = u.hi;
   s.lo += u.lo + t.lo;
 }
+// A sum carried in three floats: the TwoSum errors of hi are summed in mid, those of mid in lo.  An
+// addition loses 2^-72 of the largest partial sum, FP64 2^-53 (fp3_value rounds to FP64 once).
+struct FP3 {
+  float hi, mid, lo;
+};
+__device__ __forceinline__ void fp3_acc(FP3& s, float t) {
+  const FP u = fp_two_sum(s.hi, t), v = fp_two_sum(s.mid, u.lo);
+  s = FP3{u.hi, v.hi, s.lo + v.lo};
+}
+__device__ __forceinline__ void fp3_acc_mid(FP3& s, float t) {  // t of the size of s.mid
+  const FP v = fp_two_sum(s.mid, t);
+  s.mid = v.hi;
+  s.lo += v.lo;
+}
+__device__ __forceinline__ void fp3_acc(FP3& s, FP t) {
+  fp3_acc(s, t.hi);
+  fp3_acc_mid(s, t.lo);
+}
+__device__ __forceinline__ double fp3_value(FP3 s) { return (double)s.hi + ((double)s.mid + (double)s.lo); }
 __device__ __forceinline__ FP pair_of(float x) { return FP{x, 0.f}; }
 __device__ __forceinline__ FP pair_of(FP x) { return x; }
 

@@ -27,10 +27,10 @@
 #include <cooperative_groups.h>
 
 #include "adjoint_rc.cuh"
-#include "eft.cuh"
 #include "fft_core.cuh"
 #include "kernels.cuh"
 #include "reduce.cuh"
+#include "sums.cuh"
 #include "xy.cuh"
 
 namespace dgp {
@@ -216,43 +216,9 @@ __device__ __forceinline__ void split_store_abs(vec2_t<T>* aux, int kz, int ky, 
   if (kz == N / 2) aux[HessAux<N>::kz_nyq + (int64_t)x * N + ky] = v;
 }
 
-// Sums of a P(k) shell: sqrt(n2) and |a|^2 (/ n2^2), as float pairs for FP32 data.
-template <typename T> struct ShellSum {
-  double s = 0.0;
-  __device__ __forceinline__ void add_root(int n2, bool twice) {
-    const double r = sqrt((double)n2);
-    s += twice ? 2.0 * r : r;
-  }
-  __device__ __forceinline__ void add_norm(double2 a) { s += a.x * a.x + a.y * a.y; }
-  __device__ __forceinline__ void add_norm_over(double2 a, int n2) {
-    s += (a.x * a.x + a.y * a.y) / ((double)n2 * (double)n2);
-  }
-  __device__ __forceinline__ double value() const { return s; }
-};
-template <> struct ShellSum<float> {
-  FP s{0.f, 0.f};
-  __device__ __forceinline__ void add_root(int n2, bool twice) {
-    // sqrt(n2) = r + (n2 - r^2) / (2 r), the remainder exact (n2 < 2^24)
-    const float f = (float)n2, r = sqrtf(f);
-    float lo = fmaf(-r, r, f) / (2.f * r), hi = r;
-    if (twice) {
-      hi *= 2.f;
-      lo *= 2.f;
-    }
-    fp_acc(s, FP{hi, lo});
-  }
-  __device__ __forceinline__ void add_norm(float2 a) {
-    FP p = fp_prod(a.x, a.x);
-    fp_acc(p, fp_prod(a.y, a.y));
-    fp_acc(s, p);
-  }
-  __device__ __forceinline__ void add_norm_over(float2 a, int n2) {
-    const double q = (double)a.x * a.x + (double)a.y * a.y, v = q / ((double)n2 * (double)n2);
-    const float hi = (float)v;
-    fp_acc(s, FP{hi, (float)(v - (double)hi)});
-  }
-  __device__ __forceinline__ double value() const { return (double)s.hi + (double)s.lo; }
-};
+template <typename V> __device__ __forceinline__ double norm_d(V a) {
+  return (double)a.x * a.x + (double)a.y * a.y;
+}
 
 template <typename T, int RB> struct XBatch {
   XArgs<T> a[RB];
@@ -307,11 +273,11 @@ __global__ void __launch_bounds__(XGeom<T, N>::THREADS, XGeom<T, N>::MIN_BLOCKS)
     // Shell sums in a fixed order, so that P(k) is the same bits on every run.  Shell b holds the modes
     // with n^2 in [b^2 - b + 1, b^2 + b] (round(|n|) = b), on a column (ky, kz) one run of |kx|.  The
     // CTA's spectrum goes to shared memory and one thread per shell and half of the columns walks
-    // its runs; the halves are then added.  FP32 data sum as float pairs (about 48 bits), as the
-    // other reductions do, since FP64 instructions are what a per-mode FP64 sum waits for.
+    // its runs; the halves are then added.
     constexpr int PP = TY + 1;  // padded row: threads of neighbouring shells read neighbouring kx
     constexpr int HALVES = TY >= 2 ? 2 : 1, CPH = TY / HALVES;
-    int e = 0;  // FP32 data are scaled by 2^-e, so that their squares neither overflow nor underflow
+    int e = 0;  // FP32 data are scaled by 2^-e as they are read, so that their squares do not overflow
+    T sc = (T)1;
     if constexpr (sizeof(T) == 4) {
       __shared__ float s_max[32];
       float m = 0.f;
@@ -323,49 +289,55 @@ __global__ void __launch_bounds__(XGeom<T, N>::THREADS, XGeom<T, N>::MIN_BLOCKS)
       __syncthreads();
       for (int i = 0; i < (int)(blockDim.x + 31) / 32; ++i) m = fmaxf(m, s_max[i]);
       if (m > 0.f && isfinite(m)) e = max(ilogbf(m), -120);
-      const float sc = scalbnf(1.f, -e);
-#pragma unroll
-      for (int k2 = 0; k2 < N2; ++k2) X0[k2] = cscale(X0[k2], sc);
+      sc = scalbnf(1.f, -e);
     }
 #pragma unroll
     for (int k2 = 0; k2 < N2; ++k2) s_T[(lane + N1 * k2) * PP + yl] = X0[k2];
     __syncthreads();
     for (int i = threadIdx.x; i < HALVES * args.nbins; i += blockDim.x) {
       const int h = i / args.nbins, b = i % args.nbins + 1;
-      ShellSum<T> sk, sp, sb;
-      int cnt = 0;
-      for (int cc = 0; cc < CPH; ++cc) {
-        const int col = h * CPH + cc;
-        const int nyc = signed_index(ky0 + col, N);
-        const int r2 = nyc * nyc + nz * nz;
-        const int hi = b * b + b - r2;
-        if (hi < 0) continue;
-        int lo = b * b - b + 1 - r2;
-        if (lo < 0) lo = 0;
-        int k0 = (int)sqrtf((float)lo);  // the run |kx| = k0 .. k1 with kx^2 in [lo, hi]
-        while (k0 * k0 < lo) ++k0;
-        while (k0 > 0 && (k0 - 1) * (k0 - 1) >= lo) --k0;
-        for (int kx = k0; kx <= N / 2 && kx * kx <= hi; ++kx) {
-          const int n2 = r2 + kx * kx;
-          const V a = s_T[kx * PP + col];
-          const bool two = kx != 0 && kx != N / 2;
-          sk.add_root(n2, two);
-          sp.add_norm(a);
-          if (OP == XOP_PK_BRANE) sb.add_norm_over(a, n2);
-          ++cnt;
-          if (two) {
-            const V m = s_T[(N - kx) * PP + col];
-            sp.add_norm(m);
-            if (OP == XOP_PK_BRANE) sb.add_norm_over(m, n2);
-            ++cnt;
+      auto modes = [&](auto visit) {  // visit(n^2, two modes of opposite kx, their values)
+        for (int cc = 0; cc < CPH; ++cc) {
+          const int col = h * CPH + cc;
+          const int nyc = signed_index(ky0 + col, N);
+          const int r2 = nyc * nyc + nz * nz;
+          const int hi = b * b + b - r2;
+          if (hi < 0) continue;
+          int lo = b * b - b + 1 - r2;
+          if (lo < 0) lo = 0;
+          int k0 = (int)sqrtf((float)lo);  // the run |kx| = k0 .. k1 with kx^2 in [lo, hi]
+          while (k0 * k0 < lo) ++k0;
+          while (k0 > 0 && (k0 - 1) * (k0 - 1) >= lo) --k0;
+          for (int kx = k0; kx <= N / 2 && kx * kx <= hi; ++kx) {
+            const bool two = kx != 0 && kx != N / 2;
+            visit(r2 + kx * kx, two, s_T[kx * PP + col], s_T[(two ? N - kx : kx) * PP + col]);
           }
+        }
+      };
+      ShellSum<T> sk, sp;
+      double sb = 0.0;
+      int cnt = 0;
+      modes([&](int n2, bool two, V a, V m) {
+        sk.add_root(n2, two);
+        sp.add_norm(a.x * sc, a.y * sc);
+        if (two) sp.add_norm(m.x * sc, m.y * sc);
+        if (OP == XOP_PK_BRANE) sb += (norm_d(a) + (two ? norm_d(m) : 0.0)) / ((double)n2 * (double)n2);
+        cnt += two ? 2 : 1;
+      });
+      double p = sp.value();
+      if constexpr (sizeof(T) == 4) {
+        // a shell far below the largest mode of the CTA, or one that is not finite
+        if (cnt && !(p >= (double)kSumSmall && isfinite(p))) {
+          p = 0.0;
+          modes([&](int, bool two, V a, V m) { p += norm_d(a) + (two ? norm_d(m) : 0.0); });
+          p = scalbn(p, -2 * e);
         }
       }
       double* o = s_bins + h * NBS * args.nbins + b - 1;
       o[0] = (double)cnt;
       o[args.nbins] = sk.value();
-      o[2 * args.nbins] = sp.value();
-      if (OP == XOP_PK_BRANE) o[3 * args.nbins] = sb.value();
+      o[2 * args.nbins] = p;
+      if (OP == XOP_PK_BRANE) o[3 * args.nbins] = scalbn(sb, -2 * e);
     }
     __syncthreads();
     const double norm = scalbn(kp.box * kp.box * kp.box * kp.inv_m * kp.inv_m, 2 * e);
