@@ -8,9 +8,9 @@
 #include "common.cuh"
 #include "kernels.cuh"
 #include "cic.cuh"
-#include "eft.cuh"
 #include "reduce.cuh"
 #include "relax_control.cuh"
+#include "sums.cuh"
 
 namespace dgp {
 
@@ -272,47 +272,29 @@ void launch_sum(const T* a, int64_t m, bool absval, double* partials, int nblock
   k_sum<T><<<nblocks, 256, 0, s>>>(a, m, absval ? 1 : 0, partials);
 }
 
-// Running sum of products: FP32 factors multiply and add as float pairs (about 48 bits; FP64
-// instructions on the converted factors took 14 us a product sum at 128^3, four sums an angle),
-// FP64 factors in FP64.
-template <typename T> struct ProductSum {
-  double s = 0.0;
-  __device__ __forceinline__ void add(double a, double b) { s += a * b; }
-  __device__ __forceinline__ void add(double a, double b, double c) { s += a * b * c; }
-  __device__ __forceinline__ double value() const { return s; }
-};
-template <> struct ProductSum<float> {
-  FP s{0.f, 0.f};
-  __device__ __forceinline__ void add(float a, float b) { fp_acc(s, fp_prod(a, b)); }
-  __device__ __forceinline__ void add(float a, float b, float c) {
-    const FP p = fp_prod(a, b);
-    FP q = fp_prod(p.hi, c);
-    q.lo = fmaf(p.lo, c, q.lo);
-    fp_acc(s, q);
-  }
-  __device__ __forceinline__ double value() const { return (double)s.hi + (double)s.lo; }
-};
-
 template <typename T> struct BispecFields {
   const T* f[6];
 };
 template <typename T, bool TRIPLE>
 __global__ void __launch_bounds__(256) k_bispec_sums(const __grid_constant__ BispecFields<T> a,
-                                                     const double* __restrict__ abs_sum, int64_t m,
+                                                     const double* __restrict__ abs_sum, int64_t m, int ei,
                                                      double* __restrict__ partials) {
-  // the fields d are filtered parts of the measured field: scaled by its size, their products
-  // neither overflow nor underflow
+  // FP32: the fields d are filtered parts of the measured field, scaled by its size, the filters i are of
+  // size 1 / m
   int e = 0;
+  T sc = (T)1, si = (T)1;
   if constexpr (sizeof(T) == 4) {
-    const double mean = abs_sum[0] / (double)m;
-    if (mean > 0.0 && isfinite(mean)) e = min(max(ilogb(mean), -120), 120);
+    const float mean = (float)(abs_sum[0] / (double)m);
+    if (mean > 0.f && isfinite(mean)) e = min(max(ilogbf(mean), -120), 120);
+    sc = scalbnf(1.f, -e);
+    si = scalbnf(1.f, -ei);
   }
-  const T sc = (T)scalbn(1.0, -e);
   ProductSum<T> s0, s1, s2, s3;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
-    const T d1 = a.f[0][i] * sc, i1 = a.f[1][i], d2 = a.f[2][i] * sc, i2 = a.f[3][i];
+  const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t i = first; i < m; i += step) {
+    const T d1 = a.f[0][i] * sc, i1 = a.f[1][i] * si, d2 = a.f[2][i] * sc, i2 = a.f[3][i] * si;
     if constexpr (TRIPLE) {
-      const T d3 = a.f[4][i] * sc, i3 = a.f[5][i];
+      const T d3 = a.f[4][i] * sc, i3 = a.f[5][i] * si;
       s0.add(d1, d2, d3);
       s1.add(i1, i2, i3);
       s2.add(d3, d3);
@@ -325,11 +307,32 @@ __global__ void __launch_bounds__(256) k_bispec_sums(const __grid_constant__ Bis
     }
   }
   double v[4] = {s0.value(), s1.value(), s2.value(), s3.value()};
-  v[0] = scalbn(v[0], TRIPLE ? 3 * e : 2 * e);
-  v[2] = scalbn(v[2], 2 * e);
+  // a thread whose products are far below the scale (or not finite) adds its points in FP64
+  if (first < m && (s0.small() || s1.small() || s2.small() || s3.small())) {
+    v[0] = v[1] = v[2] = v[3] = 0.0;
+    for (int64_t i = first; i < m; i += step) {
+      const double d1 = a.f[0][i], i1 = a.f[1][i], d2 = a.f[2][i], i2 = a.f[3][i];
+      const double d3 = TRIPLE ? a.f[4][i] : d2, i3 = TRIPLE ? a.f[5][i] : i2;
+      v[0] += TRIPLE ? d1 * d2 * d3 : d1 * d1;
+      v[1] += TRIPLE ? i1 * i2 * i3 : i1 * i1;
+      v[2] += d3 * d3;
+      v[3] += i3 * i3;
+    }
+    const double p = scalbn(1.0, -e), q = scalbn(1.0, -ei);
+    v[0] = v[0] * p * p * (TRIPLE ? p : 1.0);
+    v[1] = v[1] * q * q * (TRIPLE ? q : 1.0);
+    v[2] *= p * p;
+    v[3] *= q * q;
+  }
   block_sum<4>(v);
-  if (threadIdx.x == 0)
-    for (int k = 0; k < 4; ++k) partials[4 * (int64_t)blockIdx.x + k] = v[k];
+  if (threadIdx.x == 0) {
+    double* o = partials + 4 * (int64_t)blockIdx.x;
+    const double p = sizeof(T) == 4 ? scalbn(1.0, e) : 1.0, q = sizeof(T) == 4 ? scalbn(1.0, ei) : 1.0;
+    o[0] = v[0] * p * p * (TRIPLE ? p : 1.0);
+    o[1] = v[1] * q * q * (TRIPLE ? q : 1.0);
+    o[2] = v[2] * p * p;
+    o[3] = v[3] * q * q;
+  }
 }
 
 template <typename T>
@@ -337,8 +340,9 @@ void launch_bispec_sums(T* const* f6, const double* abs_sum, int64_t m, double* 
                         cudaStream_t s) {
   BispecFields<T> a;
   for (int i = 0; i < 6; ++i) a.f[i] = f6[i];
-  if (f6[4]) k_bispec_sums<T, true><<<nblocks, 256, 0, s>>>(a, abs_sum, m, partials);
-  else k_bispec_sums<T, false><<<nblocks, 256, 0, s>>>(a, abs_sum, m, partials);
+  const int ei = sizeof(T) == 4 ? -ilogb((double)m) : 0;
+  if (f6[4]) k_bispec_sums<T, true><<<nblocks, 256, 0, s>>>(a, abs_sum, m, ei, partials);
+  else k_bispec_sums<T, false><<<nblocks, 256, 0, s>>>(a, abs_sum, m, ei, partials);
 }
 
 // delta = rho / mean - 1; FP32 data use 1 / mean as a float pair (hi + lo),

@@ -40,4 +40,32 @@ template <> struct ShellSum<float> {
   __device__ __forceinline__ double value() const { return fp3_value(s); }
 };
 
+// Sums of products of two and of three factors; small(): the products are out of the range where the
+// sum is as good as FP64.
+template <typename T> struct ProductSum {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double a, double b) { s += a * b; }
+  __device__ __forceinline__ void add(double a, double b, double c) { s += a * b * c; }
+  __device__ __forceinline__ bool small() const { return false; }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <> struct ProductSum<float> {
+  FP3 s{0.f, 0.f, 0.f};
+  float top = 0.f;  // largest product
+  __device__ __forceinline__ void add(float a, float b) {
+    const FP p = fp_prod(a, b);
+    fp3_acc(s, p);
+    top = fmaxf(top, fabsf(p.hi));
+  }
+  __device__ __forceinline__ void add(float a, float b, float c) {
+    const FP p = fp_prod(a, b), q = fp_prod(p.hi, c), r = fp_prod(p.lo, c);
+    fp3_acc(s, q);
+    fp3_acc_mid(s, r.hi);
+    s.lo += r.lo;
+    top = fmaxf(top, fabsf(q.hi));
+  }
+  __device__ __forceinline__ bool small() const { return !(top >= kSumSmall && isfinite(s.hi)); }
+  __device__ __forceinline__ double value() const { return fp3_value(s); }
+};
+
 }  // namespace dgp

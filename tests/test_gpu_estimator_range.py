@@ -34,3 +34,17 @@ def test_power_of_shells_far_below_the_largest_mode(dgp, torch_dev, n):
     finally:
         dgp.dgp_destroy(ctx)
     assert np.allclose(p / (box ** 3 * V ** 2 / n ** 6), 1.0, rtol=0, atol=1e-5)
+
+
+@pytest.mark.parametrize("n", [32, 64, 128])
+def test_bispectrum_of_shells_far_below_the_largest_mode(dgp, torch_dev, n):
+    torch, dev = torch_dev
+    box = 100.0
+    kf = 2 * math.pi / box
+    ctx = dgp.dgp_init(box, n, 1.0, OM, precision=dgp.DGP_FP32)
+    try:
+        b, q = dgp.bispectrum(ctx, _field(torch, dev, n), 3 * kf, 4 * kf, [0.3, 1.2, 2.0])
+    finally:
+        dgp.dgp_destroy(ctx)
+    assert np.allclose(b / (box ** 6 * V ** 3 / n ** 9), 1.0, rtol=0, atol=1e-5)
+    assert np.allclose(q * V * 3 / n ** 3, 1.0, rtol=0, atol=1e-5)

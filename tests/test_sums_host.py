@@ -32,6 +32,16 @@ double norm_sum(const float* x, const float* y, int n) {
   for (int i = 0; i < n; ++i) s.add_norm(x[i], y[i]);
   return s.value();
 }
+double pair_sum(const float* a, const float* b, int n) {
+  ProductSum<float> s;
+  for (int i = 0; i < n; ++i) s.add(a[i], b[i]);
+  return s.value();
+}
+double triple_sum(const float* a, const float* b, const float* c, int n) {
+  ProductSum<float> s;
+  for (int i = 0; i < n; ++i) s.add(a[i], b[i], c[i]);
+  return s.value();
+}
 }
 """
 
@@ -82,3 +92,12 @@ def test_norm_sum(lib, n, spread):
     x, y = _floats(n, n, spread), _floats(n + 1, n, spread)
     terms = [Fraction(float(a)) ** 2 + Fraction(float(b)) ** 2 for a, b in zip(x, y)]
     _check(_call(lib, "norm_sum", x, y), terms)
+
+
+@pytest.mark.parametrize("n", [1, 7, 900, 8000])
+@pytest.mark.parametrize("spread", [0, 12])
+def test_product_sums(lib, n, spread):
+    a, b, c = (_floats(n + i, n, spread) for i in range(3))
+    f = [[Fraction(float(v)) for v in x] for x in (a, b, c)]
+    _check(_call(lib, "pair_sum", a, b), [x * y for x, y, _ in zip(*f)])
+    _check(_call(lib, "triple_sum", a, b, c), [x * y * z for x, y, z in zip(*f)])
