@@ -447,24 +447,6 @@ __device__ __forceinline__ T block_mean_d(const double* dsum, int64_t m) {
   return s_mean;
 }
 
-// A thread's sums: float pairs for FP32 data (FP64 additions of converted values bound these passes
-// to the FP64 pipe), FP64 otherwise.
-template <typename T> struct ThreadSum {
-  double s = 0.0;
-  __device__ __forceinline__ void add(double v) { s += v; }
-  __device__ __forceinline__ void add_inverse(double v) { s += 1.0 / v; }
-  __device__ __forceinline__ double value() const { return s; }
-};
-template <> struct ThreadSum<float> {
-  FP s{0.f, 0.f};
-  __device__ __forceinline__ void add(float v) { fp_acc(s, FP{v, 0.f}); }
-  __device__ __forceinline__ void add_inverse(float v) {  // 1 / v = r + r (1 - r v), the remainder exact
-    const float r = 1.f / v;
-    fp_acc(s, FP{r, r * fmaf(-r, v, 1.f)});
-  }
-  __device__ __forceinline__ double value() const { return (double)s.hi + (double)s.lo; }
-};
-
 template <typename T>
 __global__ void __launch_bounds__(256) k_adj_update_a(const T* __restrict__ lam, const T* __restrict__ D,
                                                       const double* __restrict__ dsum, const T* __restrict__ g,

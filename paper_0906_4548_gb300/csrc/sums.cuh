@@ -40,6 +40,26 @@ template <> struct ShellSum<float> {
   __device__ __forceinline__ double value() const { return fp3_value(s); }
 };
 
+// Sums of values and of their inverses.
+template <typename T> struct ThreadSum {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double v) { s += v; }
+  __device__ __forceinline__ void add_inverse(double v) { s += 1.0 / v; }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <> struct ThreadSum<float> {
+  FP3 s{0.f, 0.f, 0.f};
+  __device__ __forceinline__ void add(float v) { fp3_acc(s, v); }
+  __device__ __forceinline__ void add_inverse(float v) {
+    // 1 / v = r (1 + t + t^2 + ...), t = 1 - r v exactly, |t| < 2^-23
+    const float r = 1.f / v, t = fmaf(-r, v, 1.f);
+    const FP p = fp_prod(r, t);
+    fp3_acc(s, FP{r, p.hi});
+    s.lo += fmaf(r * t, t, p.lo);
+  }
+  __device__ __forceinline__ double value() const { return fp3_value(s); }
+};
+
 // Sums of products of two and of three factors; small(): the products are out of the range where the
 // sum is as good as FP64.
 template <typename T> struct ProductSum {

@@ -32,6 +32,16 @@ double norm_sum(const float* x, const float* y, int n) {
   for (int i = 0; i < n; ++i) s.add_norm(x[i], y[i]);
   return s.value();
 }
+double value_sum(const float* x, int n) {
+  ThreadSum<float> s;
+  for (int i = 0; i < n; ++i) s.add(x[i]);
+  return s.value();
+}
+double inverse_sum(const float* x, int n) {
+  ThreadSum<float> s;
+  for (int i = 0; i < n; ++i) s.add_inverse(x[i]);
+  return s.value();
+}
 double pair_sum(const float* a, const float* b, int n) {
   ProductSum<float> s;
   for (int i = 0; i < n; ++i) s.add(a[i], b[i]);
@@ -101,3 +111,11 @@ def test_product_sums(lib, n, spread):
     f = [[Fraction(float(v)) for v in x] for x in (a, b, c)]
     _check(_call(lib, "pair_sum", a, b), [x * y for x, y, _ in zip(*f)])
     _check(_call(lib, "triple_sum", a, b, c), [x * y * z for x, y, z in zip(*f)])
+
+
+@pytest.mark.parametrize("n", [1, 7, 900, 8000])
+@pytest.mark.parametrize("spread", [0, 12])
+def test_value_and_inverse_sums(lib, n, spread):
+    x = _floats(n + 5, n, spread)
+    _check(_call(lib, "value_sum", x), [Fraction(float(v)) for v in x])
+    _check(_call(lib, "inverse_sum", x), [1 / Fraction(float(v)) for v in x])
