@@ -282,7 +282,8 @@ __global__ void __launch_bounds__(RowGeom<N, RowWide<N, AR, RB>::W>::THREADS, Ro
   uint64_t* bars = reinterpret_cast<uint64_t*>(s_tw + N);        // [2]
   double* s_part = reinterpret_cast<double*>(bars + 2);          // [4][WARPS]
   double* s_mean = s_part + 4 * WARPS;                           // mean, then its float pair
-  int* s_cnt = reinterpret_cast<int*>(s_mean + 2);               // arrivals: A read, B read, done; then a wait gave up
+  // arrivals (A read, B read, done), then flags: a wait gave up, C issued, the rows issued
+  int* s_cnt = reinterpret_cast<int*>(s_mean + 2);
   const int tid = threadIdx.x, wid = tid >> 5, wl = tid & 31;
   const int c = (wl >> 1) % N2, r = wid * (32 / N2) + 2 * ((wl >> 1) / N2) + (wl & 1);
   const int x = blockIdx.y, y0 = blockIdx.x * TY;
@@ -309,7 +310,7 @@ __global__ void __launch_bounds__(RowGeom<N, RowWide<N, AR, RB>::W>::THREADS, Ro
     float* mp = reinterpret_cast<float*>(s_mean + 1);
     mp[0] = (float)m;
     mp[1] = (float)(m - (double)mp[0]);
-    s_cnt[0] = s_cnt[1] = s_cnt[2] = s_cnt[3] = 0;
+    for (int i = 0; i < 6; ++i) s_cnt[i] = 0;
   }
   for (int i = tid; i < N; i += G::THREADS) s_tw[i] = g_tw[(RowSplit<N, WIDE>::PHASES ? N : 0) + i];
   __syncthreads();
@@ -349,7 +350,10 @@ __global__ void __launch_bounds__(RowGeom<N, RowWide<N, AR, RB>::W>::THREADS, Ro
   row_pair_inverse<N, WIDE>(buf0, s_tw, r, c, ra, rb);
 #pragma unroll
   for (int i = 0; i < PTS; ++i) AR::pair_a(acc[i], ra[i], rb[i]);
-  if (last_warp(0) && wl == 0 && !gave_up()) issue(buf0, 0, 1, &bars[0]);  // pair C, the diagonal
+  if (last_warp(0) && wl == 0 && !gave_up()) {  // pair C, the diagonal
+    s_cnt[4] = 1;
+    issue(buf0, 0, 1, &bars[0]);
+  }
   wait(&bars[1], 0);
   row_pair_inverse<N, WIDE>(buf1, s_tw, r, c, ra, rb);
 #pragma unroll
@@ -357,8 +361,12 @@ __global__ void __launch_bounds__(RowGeom<N, RowWide<N, AR, RB>::W>::THREADS, Ro
   float* sD = reinterpret_cast<float*>(buf1);
   float* sS = sD + TY * ROWP;
   const int64_t rbase0 = ((int64_t)x * N + y0) * N;
-  if (last_warp(1) && !gave_up()) {  // the rows of D and S
-    if (wl == 0) mbar_expect_tx(&bars[1], 2u * TY * N * 4);
+  // the rows of D and S; the flag may be set meanwhile, so one answer for the warp
+  if (last_warp(1) && !__any_sync(0xffffffffu, gave_up())) {
+    if (wl == 0) {
+      s_cnt[5] = 1;
+      mbar_expect_tx(&bars[1], 2u * TY * N * 4);
+    }
     __syncwarp();
     const float* src = (wl < TY ? args.D : args.S) + rbase0 + (int64_t)(wl % TY) * N;
     bulk_load((wl < TY ? sD : sS) + (wl % TY) * ROWP, src, N * 4, &bars[1]);
@@ -439,11 +447,13 @@ __global__ void __launch_bounds__(RowGeom<N, RowWide<N, AR, RB>::W>::THREADS, Ro
   }
   if (wl == 0) {
     if (gave_up()) {
-      // the copies that were issued: B, and A unless withheld; C and the rows only without a fault
-      // so far, and then their phases are waited for as well (bounded; a phase with no copy runs out)
-      const uint64_t lim2 = 4 * lim + 1000000ull;
-      if (!args.withhold) mbar_wait_bounded(&bars[0], 0, lim2) && mbar_wait_bounded(&bars[0], 1, lim2);
-      mbar_wait_bounded(&bars[1], 0, lim2) && mbar_wait_bounded(&bars[1], 1, lim2);
+      // every copy issued lands, or this wait runs out too, before the CTA's shared memory is given back:
+      // C and the rows are issued only once the phase before them has completed (bounded; nothing waits
+      // for a copy that was not issued)
+      const uint64_t lim2 = 4 * lim + 1000000000ull;
+      if (s_cnt[4]) mbar_wait_bounded(&bars[0], 1, lim2);
+      else if (!args.withhold) mbar_wait_bounded(&bars[0], 0, lim2);
+      mbar_wait_bounded(&bars[1], s_cnt[5] ? 1 : 0, lim2);
       return;
     }
 #pragma unroll

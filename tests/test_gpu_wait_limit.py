@@ -6,6 +6,8 @@ and the solve reports DGP_E_TIMEOUT.  The test makes a wait run out without any 
 the test hook leaves one copy unissued (so its barrier is never completed), with a 1 ms bound.
 The context must then solve normally again, to the oracle's phi.
 """
+import time
+
 import numpy as np
 import pytest
 
@@ -54,3 +56,32 @@ def test_wait_limit_rejects_bad_bounds(dgp, torch_dev):
             assert e.value.status == dgp.DGP_E_INVALID
     finally:
         dgp.dgp_destroy(ctx)
+
+
+@pytest.mark.parametrize("n,prec", [(32, "DGP_MIXED_EFT"), (48, "DGP_FP32"), (64, "DGP_MIXED_EFT"), (96, "DGP_MIXED")])
+def test_fault_waits_for_no_copy_that_was_not_issued(dgp, torch_dev, n, prec):
+    """Before it returns, a CTA whose wait ran out waits (up to four limits and a second) for the copies it
+    issued.  All of them land here but the withheld one, so the solve ends after one limit for each wave of CTAs
+    (one wave up to 64^3, two at 96^3), not after five."""
+    torch, dev = torch_dev
+    limit, waves = 0.3, 2 if n == 96 else 1
+    ctx = dgp.dgp_init(2.0 * n, n, 1.0, OM, precision=getattr(dgp, prec))
+    try:
+        g = torch.Generator(device=dev)
+        g.manual_seed(n)
+        d = torch.rand((n, n, n), generator=g, device=dev) - 0.5
+        dgp.dgp_solve_phi(ctx, 0.5, d, None, 1e-3)  # the kernels are loaded
+        dgp.dgp_reset(ctx)
+        dgp.dgp_set_wait_limit(ctx, limit, True)
+        torch.cuda.synchronize()
+        t = time.perf_counter()
+        with pytest.raises(dgp.DgpError) as e:
+            dgp.dgp_solve_phi(ctx, 0.5, d, None, 1e-3)
+        t = time.perf_counter() - t
+        assert e.value.status == dgp.DGP_E_TIMEOUT
+        dgp.dgp_set_wait_limit(ctx, 2.0, False)
+        st, _ = dgp.dgp_solve_phi(ctx, 0.5, d, None, 1e-3)
+        assert st == dgp.DGP_OK
+    finally:
+        dgp.dgp_destroy(ctx)
+    assert limit <= t < (waves + 1.5) * limit
