@@ -361,7 +361,10 @@ class Engine : public EngineBase {
   SolveCtl* d_ctl = nullptr;    // stop-rule state of the running solve
   SolveCtl* h_ctl = nullptr;    // pinned host copy
   double* d_hist = nullptr;     // [max_iter + 1] normalised residuals of the running solve
-  double* h_hist = nullptr;     // pinned host copy, read with the verdict
+  // pinned host copy of the first residuals, read with the verdict; a solve of more evaluations (few take
+  // more than 40) reads the rest when it has ended, so that a large max_iter pins no memory
+  static constexpr int kPinnedHist = 64;
+  double* h_hist = nullptr;
   int last_stop_it = -1;        // last iteration examined by the previous solve
   double last_nl_a = -1.0;      // scale factor of the last nonlinear solve
   static constexpr int kPatience = 10;  // iterations without a new minimum before stopping
@@ -457,7 +460,7 @@ class Engine : public EngineBase {
     if (cudaMalloc(&d_ctl, sizeof(SolveCtl)) != cudaSuccess) return DGP_E_NOMEM;
     if (cudaMallocHost(&h_ctl, sizeof(SolveCtl)) != cudaSuccess) return DGP_E_NOMEM;
     if (cudaMalloc(&d_hist, sizeof(double) * ((size_t)p.max_iter + 1)) != cudaSuccess) return DGP_E_NOMEM;
-    if (cudaMallocHost(&h_hist, sizeof(double) * ((size_t)p.max_iter + 1)) != cudaSuccess) return DGP_E_NOMEM;
+    if (cudaMallocHost(&h_hist, sizeof(double) * kPinnedHist) != cudaSuccess) return DGP_E_NOMEM;
     pk_blocks = x_pass_blocks<T, N>();
     if (cudaMalloc(&pk_partials, sizeof(double) * 4 * (N / 2) * (size_t)pk_blocks) != cudaSuccess) return DGP_E_NOMEM;
     if (cudaMalloc(&d_pk, sizeof(double) * 4 * (N / 2)) != cudaSuccess) return DGP_E_NOMEM;
@@ -802,8 +805,7 @@ class Engine : public EngineBase {
           }
         }
         DGP_CUDA(cudaMemcpyAsync(h_ctl, d_ctl, sizeof(SolveCtl), cudaMemcpyDeviceToHost, stream));
-        DGP_CUDA(cudaMemcpyAsync(h_hist, d_hist, sizeof(double) * std::min(it, p.max_iter + 1), cudaMemcpyDeviceToHost,
-                                 stream));
+        DGP_CUDA(cudaMemcpyAsync(h_hist, d_hist, sizeof(double) * pinned_hist(it), cudaMemcpyDeviceToHost, stream));
         DGP_CUDA(wait_stream());
         if (h_ctl->done || it > p.max_iter) break;
         chunk = kChunk;
@@ -812,7 +814,7 @@ class Engine : public EngineBase {
       if (!st.done) return DGP_E_STATE;  // the controller stops at it = max_iter at the latest
       const int s_it = st.stop_it;
       credit(s_it + 1, s_it);
-      history.assign(h_hist, h_hist + s_it + 1);
+      if ((rc = keep_history(s_it + 1))) return rc;
       if (st.status == CTL_FAULT) return DGP_E_TIMEOUT;
       if (st.status == CTL_NONFINITE) return DGP_E_NONFINITE;
       last_stop_it = s_it;
@@ -875,6 +877,23 @@ class Engine : public EngineBase {
       DGP_CUDA(wait_stream());
     }
     return status;
+  }
+
+  // how many of the first `evaluations` residuals (at most max_iter + 1) the pinned copy holds
+  int pinned_hist(int evaluations) const {
+    return (int)std::min({(int64_t)evaluations, (int64_t)p.max_iter + 1, (int64_t)kPinnedHist});
+  }
+  // history <- the residuals of an ended solve, whose first ones the verdict has brought
+  int keep_history(int evaluations) {
+    const int first = pinned_hist(evaluations);
+    history.assign(h_hist, h_hist + first);
+    if (evaluations > first) {
+      history.resize(evaluations);
+      DGP_CUDA(cudaMemcpyAsync(history.data() + first, d_hist + first, sizeof(double) * (evaluations - first),
+                               cudaMemcpyDeviceToHost, stream));
+      DGP_CUDA(wait_stream());
+    }
+    return DGP_OK;
   }
 
   CicParams cic() const {
@@ -1196,7 +1215,7 @@ class Engine : public EngineBase {
       if (!plane) pf.run(KK_Y, 2 * nS, st, [&] { launch_fft_y_batch<T, N>(f, nullptr, nullptr, n, 1, false, tw, st, yt); });
     }
     VerdictBatch vb;
-    for (int k = 0; k < n; ++k) vb.m[k] = {S[k]->d_ctl, S[k]->d_hist, S[k]->h_ctl, S[k]->h_hist, S[k]->p.max_iter + 1};
+    for (int k = 0; k < n; ++k) vb.m[k] = {S[k]->d_ctl, S[k]->d_hist, S[k]->h_ctl, S[k]->h_hist, S[k]->pinned_hist(kPinnedHist)};
     launch_clear_verdicts(vb, n, st);
     int rc;
     if ((rc = check())) return rc;
@@ -1344,7 +1363,7 @@ class Engine : public EngineBase {
     for (int k = 0; k < n; ++k) {
       ctl[k] = *S[k]->h_ctl;
       if (!ctl[k].done) return DGP_E_STATE;
-      S[k]->history.assign(S[k]->h_hist, S[k]->h_hist + ctl[k].stop_it + 1);
+      if ((rc = S[k]->keep_history(ctl[k].stop_it + 1))) return rc;
     }
     std::vector<V*> sDphi(n);
     FieldSet<T> fy[kBatchMax];  // plane pass: accepted spectra still to be transformed along y
