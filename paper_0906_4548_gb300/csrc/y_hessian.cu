@@ -50,7 +50,10 @@ template <typename T, int N> struct YHGeom {
   static constexpr bool SPLIT = CTAS <= 304;
   static constexpr int OUTS = SPLIT ? 3 : 1;
   static constexpr size_t SMEM = sizeof(vec2_t<T>) * (N + (SPLIT ? 3 : 2) * (size_t)P * RS);
-  static constexpr int MINB = sizeof(T) == 8 ? 1 : N == 512 ? 5 : SPLIT ? 1 : 512 / THREADS;
+  // FP64 at 48^3, 384 threads: registers for two CTAs, since one CTA with the whole register file shuts out
+  // the contexts that run beside it (six of them stepping: 12.45 -> 11.65 ms, with the passes before the
+  // split 11.95; one alone: 3.37 -> 3.27 ms)
+  static constexpr int MINB = sizeof(T) == 8 ? (SPLIT ? 2 : 1) : N == 512 ? 5 : SPLIT ? 1 : 512 / THREADS;
   static_assert(N % P == 0, "a CTA's rows share kz");
 };
 
