@@ -116,14 +116,12 @@ template <int N, bool WIDE> __device__ __forceinline__ float2 row_phase(const fl
 template <int N, bool WIDE>
 using RowSlots = TileSlots<RowGeom<N, WIDE>::N1, RowGeom<N, WIDE>::N2, RowGeom<N, WIDE>::FIELD - (N / 2) * 128>;
 
-// Inverse z transform of the pair in buf: on return a[i], b[i] with i = q + Q k2 are the two fields at
-// z = k1 + N1 k2, k1 = c + N2 q (zero where k1 >= N1); z = c + N2 i when EVEN.
+// First stage of the inverse z transform of the pair in buf, its transpose in the row's slots.
 template <int N, bool WIDE>
-__device__ __forceinline__ void row_pair_inverse(unsigned char* buf, const float2* s_tw, int r, int c,
-                                                 float (&a)[RowGeom<N, WIDE>::PTS], float (&b)[RowGeom<N, WIDE>::PTS]) {
+__device__ __forceinline__ void row_pair_first(unsigned char* buf, const float2* s_tw, int r, int c) {
   using G = RowGeom<N, WIDE>;
   using S = RowSlots<N, WIDE>;
-  constexpr int N1 = G::N1, N2 = G::N2, Q = G::Q;
+  constexpr int N1 = G::N1, N2 = G::N2;
   {
     float2 v[N1];
     const unsigned char* TA = buf;
@@ -154,33 +152,60 @@ __device__ __forceinline__ void row_pair_inverse(unsigned char* buf, const float
       tile_at(buf, S::by_col(off_d, k1)) = k1 == 0 ? v[k1] : cmul(v[k1], row_phase<N, WIDE>(s_tw, k1, c));
   }
   __syncwarp();
+}
+
+// The two fields (a, -b) of sample z = c + N2 i after row_pair_to_slots.
+template <int N, bool WIDE>
+__device__ __forceinline__ float2 row_pair_sample(const unsigned char* buf, int r, int c, int i) {
+  return tile_at(buf, RowSlots<N, WIDE>::folded(c + RowGeom<N, WIDE>::N2 * i, r));
+}
+
+// Inverse z transform of the pair in buf: rows k1 on the lanes that have one, then sample z to the slot
+// of line z.
+template <int N, bool WIDE>
+__device__ __forceinline__ void row_pair_to_slots(unsigned char* buf, const float2* s_tw, int r, int c) {
+  using G = RowGeom<N, WIDE>;
+  using S = RowSlots<N, WIDE>;
+  constexpr int N1 = G::N1, N2 = G::N2, Q = G::Q;
+  row_pair_first<N, WIDE>(buf, s_tw, r, c);
+  float2 u[Q][N2];
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    if (c + N2 * q >= N1) continue;
+    const int base = S::by_row_base(c + N2 * q, r);
+#pragma unroll
+    for (int j2 = 0; j2 < N2; ++j2) u[q][j2] = tile_at(buf, S::by_row(base, j2));
+    dft_regs<N2, N / N2>(u[q], s_tw);
+  }
+  __syncwarp();
+#pragma unroll
+  for (int q = 0; q < Q; ++q) {
+    if (c + N2 * q >= N1) continue;
+#pragma unroll
+    for (int k2 = 0; k2 < N2; ++k2) tile_at(buf, S::folded(c + N2 * q + N1 * k2, r)) = u[q][k2];
+  }
+  __syncwarp();
+}
+
+// Inverse z transform of the pair in buf: on return a[i], b[i] with i = q + Q k2 are the two fields at
+// z = k1 + N1 k2, k1 = c + N2 q (zero where k1 >= N1); z = c + N2 i when EVEN.
+template <int N, bool WIDE>
+__device__ __forceinline__ void row_pair_inverse(unsigned char* buf, const float2* s_tw, int r, int c,
+                                                 float (&a)[RowGeom<N, WIDE>::PTS], float (&b)[RowGeom<N, WIDE>::PTS]) {
+  using G = RowGeom<N, WIDE>;
+  using S = RowSlots<N, WIDE>;
+  constexpr int N1 = G::N1, N2 = G::N2, Q = G::Q;
   if constexpr (WIDE) {
-    // rows k1 on the lanes that have one; then sample z to the slot of line z, and lane c takes its column
-    float2 u[Q][N2];
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      if (c + N2 * q >= N1) continue;
-      const int base = S::by_row_base(c + N2 * q, r);
-#pragma unroll
-      for (int j2 = 0; j2 < N2; ++j2) u[q][j2] = tile_at(buf, S::by_row(base, j2));
-      dft_regs<N2, N / N2>(u[q], s_tw);
-    }
-    __syncwarp();
-#pragma unroll
-    for (int q = 0; q < Q; ++q) {
-      if (c + N2 * q >= N1) continue;
-#pragma unroll
-      for (int k2 = 0; k2 < N2; ++k2) tile_at(buf, S::folded(c + N2 * q + N1 * k2, r)) = u[q][k2];
-    }
-    __syncwarp();
+    row_pair_to_slots<N, WIDE>(buf, s_tw, r, c);
 #pragma unroll
     for (int i = 0; i < N1; ++i) {
-      const float2 v = tile_at(buf, S::folded(c + N2 * i, r));
+      const float2 v = row_pair_sample<N, WIDE>(buf, r, c, i);
       a[i] = v.x;
       b[i] = -v.y;
     }
     return;
   }
+  row_pair_first<N, WIDE>(buf, s_tw, r, c);
 #pragma unroll
   for (int q = 0; q < Q; ++q) {
     if (!G::EVEN && c + N2 * q >= N1) {
@@ -263,6 +288,13 @@ template <int N, class AR, int RB> struct RowWide {
   static constexpr bool F64 = std::is_same<typename AR::Sum, double>::value;
   static constexpr bool EFT = std::is_same<AR, RxEFT>::value;
   static constexpr bool W = (N == 32 || N == 48 || N == 96) && (F64 || (RB == 1 && (EFT || N == 48)));
+  // Float pairs at 512^3, 32 points to a lane: unrolled over them the arithmetic alone is some 56 KB of
+  // code, which 8 warps an SM wait for.  The points go in a rolled loop then, their fields through the row's
+  // slots and the accumulators through shared memory: 3989 -> 2335 us a launch (2523 with rows spread over
+  // the CTA).
+  static constexpr bool ROLL = N == 512 && EFT;
+  using G = RowGeom<N, W>;
+  static constexpr size_t SMEM = G::SMEM + (ROLL ? sizeof(float2) * G::THREADS * G::PTS : 0);
 };
 
 template <int N, class AR, int RB>
@@ -270,7 +302,7 @@ __global__ void __launch_bounds__(RowGeom<N, RowWide<N, AR, RB>::W>::THREADS, Ro
     k_relax_rows(const __grid_constant__ RelaxTmaBatch<RB> batch, const float2* __restrict__ g_tw) {
   const RelaxTmaArgs& args = batch.a[RB > 1 ? blockIdx.z : 0];  // realisation of this CTA
   if (args.skip && *args.skip) return;
-  constexpr bool WIDE = RowWide<N, AR, RB>::W;
+  constexpr bool WIDE = RowWide<N, AR, RB>::W, ROLL = RowWide<N, AR, RB>::ROLL;
   using G = RowGeom<N, WIDE>;
   using Acc = typename AR::Acc;
   using Sum = typename AR::Sum;
@@ -343,21 +375,44 @@ __global__ void __launch_bounds__(RowGeom<N, RowWide<N, AR, RB>::W>::THREADS, Ro
   };
   auto gave_up = [&]() { return *reinterpret_cast<volatile int*>(&s_cnt[3]) != 0; };
 
-  constexpr int PTS = G::PTS, Q = G::Q;
-  Acc acc[PTS];
-  float ra[PTS], rb[PTS];
+  constexpr int PTS = G::PTS, Q = G::Q, HELD = ROLL ? 1 : PTS;
+  Acc acc[HELD];
+  float ra[HELD], rb[HELD];
+  // ROLL: the thread's accumulators, [point][thread]
+  float2* s_acc = reinterpret_cast<float2*>(s_cnt + 8) + tid;
   wait(&bars[0], 0);
-  row_pair_inverse<N, WIDE>(buf0, s_tw, r, c, ra, rb);
+  if constexpr (ROLL) {
+    row_pair_to_slots<N, WIDE>(buf0, s_tw, r, c);
+#pragma unroll 4
+    for (int i = 0; i < PTS; ++i) {
+      const float2 v = row_pair_sample<N, WIDE>(buf0, r, c, i);
+      AR::pair_a(acc[0], v.x, -v.y);
+      s_acc[i * G::THREADS] = make_float2(acc[0].hi, acc[0].lo);
+    }
+  } else {
+    row_pair_inverse<N, WIDE>(buf0, s_tw, r, c, ra, rb);
 #pragma unroll
-  for (int i = 0; i < PTS; ++i) AR::pair_a(acc[i], ra[i], rb[i]);
+    for (int i = 0; i < PTS; ++i) AR::pair_a(acc[i], ra[i], rb[i]);
+  }
   if (last_warp(0) && wl == 0 && !gave_up()) {  // pair C, the diagonal
     s_cnt[4] = 1;
     issue(buf0, 0, 1, &bars[0]);
   }
   wait(&bars[1], 0);
-  row_pair_inverse<N, WIDE>(buf1, s_tw, r, c, ra, rb);
+  if constexpr (ROLL) {
+    row_pair_to_slots<N, WIDE>(buf1, s_tw, r, c);
+#pragma unroll 4
+    for (int i = 0; i < PTS; ++i) {
+      const float2 v = row_pair_sample<N, WIDE>(buf1, r, c, i), t = s_acc[i * G::THREADS];
+      acc[0] = Acc{t.x, t.y};
+      AR::pair_b(acc[0], v.x, -v.y, rp);
+      s_acc[i * G::THREADS] = make_float2(acc[0].hi, acc[0].lo);
+    }
+  } else {
+    row_pair_inverse<N, WIDE>(buf1, s_tw, r, c, ra, rb);
 #pragma unroll
-  for (int i = 0; i < PTS; ++i) AR::pair_b(acc[i], ra[i], rb[i], rp);
+    for (int i = 0; i < PTS; ++i) AR::pair_b(acc[i], ra[i], rb[i], rp);
+  }
   float* sD = reinterpret_cast<float*>(buf1);
   float* sS = sD + TY * ROWP;
   const int64_t rbase0 = ((int64_t)x * N + y0) * N;
@@ -372,19 +427,17 @@ __global__ void __launch_bounds__(RowGeom<N, RowWide<N, AR, RB>::W>::THREADS, Ro
     bulk_load((wl < TY ? sD : sS) + (wl % TY) * ROWP, src, N * 4, &bars[1]);
   }
   wait(&bars[0], 1);
-  row_pair_inverse<N, WIDE>(buf0, s_tw, r, c, ra, rb);  // a, b: two diagonal second derivatives
+  // a, b: two diagonal second derivatives
+  if constexpr (ROLL) row_pair_to_slots<N, WIDE>(buf0, s_tw, r, c);
+  else row_pair_inverse<N, WIDE>(buf0, s_tw, r, c, ra, rb);
   wait(&bars[1], 1);
   Sum rsum{};
   FP acc_d{0.f, 0.f};  // sum of D_new: its mean is removed next iteration
   float nbad = 0.f, nonfin = 0.f;
   float* dst = args.Dnew + rbase0 + (int64_t)r * N;
-#pragma unroll
-  for (int i = 0; i < PTS; ++i) {
-    const int k1 = c + N2 * (i % Q);
-    if (!G::EVEN && k1 >= N1) continue;
-    const int z = G::EVEN ? c + N2 * i : k1 + N1 * (i / Q);
-    const PointOut o = AR::finish(acc[i], ra[i], rb[i], sD[r * ROWP + z], sS[r * ROWP + z], m_hi, m_lo, mean, rp,
-                                  rsum, nonfin);
+  // residual and update at sample z, which returns D_new
+  auto update = [&](Acc& t, float fa, float fb, int z) {
+    const PointOut o = AR::finish(t, fa, fb, sD[r * ROWP + z], sS[r * ROWP + z], m_hi, m_lo, mean, rp, rsum, nonfin);
     float bpt = o.bp, dt = o.dt;
     if (o.neg) {
       nbad += 1.f;
@@ -400,13 +453,32 @@ __global__ void __launch_bounds__(RowGeom<N, RowWide<N, AR, RB>::W>::THREADS, Ro
       dn = 2.f * bpt / (rp.alpha_f + sqrtf(dt));
     }
     dst[z] = dn;
-    if constexpr (G::EVEN) ra[i] = dn;
-    else sD[r * ROWP + z] = dn;
     if constexpr (std::is_same<AR, RxF32>::value) acc_d.hi += dn;
     else fp_acc(acc_d, FP{dn, 0.f});
+    return dn;
+  };
+  constexpr bool VIA_SD = ROLL || !G::EVEN;  // D_new reaches the forward transform's lanes through sD
+  if constexpr (ROLL) {
+#pragma unroll 2
+    for (int i = 0; i < PTS; ++i) {
+      const float2 v = row_pair_sample<N, WIDE>(buf0, r, c, i), t = s_acc[i * G::THREADS];
+      acc[0] = Acc{t.x, t.y};
+      const int z = c + N2 * i;
+      sD[r * ROWP + z] = update(acc[0], v.x, -v.y, z);
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < PTS; ++i) {
+      const int k1 = c + N2 * (i % Q);
+      if (!G::EVEN && k1 >= N1) continue;
+      const int z = G::EVEN ? c + N2 * i : k1 + N1 * (i / Q);
+      const float dn = update(acc[i], ra[i], rb[i], z);
+      if constexpr (VIA_SD) sD[r * ROWP + z] = dn;
+      else ra[i] = dn;
+    }
   }
   __syncwarp();  // the row's slots of buf0 are read, its D_new is written
-  if constexpr (G::EVEN) {
+  if constexpr (!VIA_SD) {
     row_forward<N, WIDE>(buf0, s_tw, r, c, ra);
   } else {
     float d[N1];

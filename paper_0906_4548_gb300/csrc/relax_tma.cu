@@ -267,9 +267,10 @@ template <int N, class AR, int RB>
 static void launch_rt(const RelaxTmaArgs* a, int count, const float2* tw, cudaStream_t s) {
   RelaxTmaBatch<RB> b;
   for (int r = 0; r < count; ++r) b.a[r] = a[r];
-  using G = RowGeom<N, RowWide<N, AR, RB>::W>;
-  raise_smem_limit<k_relax_rows<N, AR, RB>>(G::SMEM);
-  k_relax_rows<N, AR, RB><<<dim3(N / G::TY, N, count), G::THREADS, G::SMEM, s>>>(b, tw);
+  using W = RowWide<N, AR, RB>;
+  using G = typename W::G;
+  raise_smem_limit<k_relax_rows<N, AR, RB>>(W::SMEM);
+  k_relax_rows<N, AR, RB><<<dim3(N / G::TY, N, count), G::THREADS, W::SMEM, s>>>(b, tw);
 }
 
 template <int N, class AR>
