@@ -490,13 +490,12 @@ class Engine : public EngineBase {
   // Tile autotuning: time the y pass's CTA sizes (128, 256, 512 threads; 128 / N1,
   // ... rows per CTA) on the launch that every relaxation iteration makes, the
   // forward transform of one field with the CTA of the stop rules (whose sum over
-  // the block partials is what a 256^3 launch of 128 threads waits for), over this
-  // context's six spectrum buffers in turn, and keep the fastest.  A larger CTA has
+  // the block partials is what a 256^3 launch of 128 threads waits for), over
+  // several of this context's spectrum buffers, and keep the fastest.  A larger CTA has
   // to be faster by 3 %: the launches of a small mesh scatter by that.  The results
   // do not depend on the choice (every row's arithmetic is the same).
   int tune_tiles() {
     for (int i = 0; i < 6; ++i) DGP_CUDA(cudaMemsetAsync(s6[i], 0, sizeof(V) * SPEC, stream));
-    DGP_CUDA(cudaMemsetAsync(partials, 0, sizeof(double) * 4 * fblocks, stream));
     DGP_CUDA(cudaMemsetAsync(d_ctl, 1, sizeof(SolveCtl), stream));  // a solve that is done: no rule is applied
     const YControl yc{partials, fblocks, d_misc + 4, d_ctl, d_misc + 1, d_hist, p.max_iter,
                       kPatience, p.tol, 1.0 / (double)M};
@@ -515,7 +514,7 @@ class Engine : public EngineBase {
     for (int c = 0; c < 3 && rc == DGP_OK; ++c) {
       pass(0, cand[c]);  // warm-up
       cudaEventRecord(e0, stream);
-      for (int r = 0; r < 18; ++r) pass(r % 6, cand[c]);
+      for (int r = 1; r < 4; ++r) pass(r, cand[c]);
       cudaEventRecord(e1, stream);
       float ms = 0.f;
       if (cudaEventSynchronize(e1) != cudaSuccess || cudaEventElapsedTime(&ms, e0, e1) != cudaSuccess ||
