@@ -305,9 +305,10 @@ int dgp_time_factors(const dgp_cosmology *cosmo, double rc_H0, double a0, double
  *   base:      at dgp_init (14 real fields, 9 half spectra, twiddles, reduction
  *              partials, residual history);
  *   sort:      added by the first dgp_sort_particles / sorting pm_step of np
- *              particles (keys, six permuted arrays, three int32 fields per cell);
- *   adjoint:   added by the first pm_step_adjoint of np particles (products,
- *              spectra, cotangent grids, the recomputed particle state);
+ *              particles (keys, records of a particle's six values, three int32
+ *              fields per cell);
+ *   adjoint:   added by the first pm_step_adjoint of np particles (lam, spectra,
+ *              cotangent grids, the recomputed particle state);
  *   host_step: added by the first pm_step_host of np particles.
  * The reduction partials depend on the device's SM count (1 when no device is
  * visible; a few KB either way).  Only p->n, p->precision and p->max_iter are

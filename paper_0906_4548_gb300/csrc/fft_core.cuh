@@ -146,7 +146,7 @@ template <typename V> __device__ __forceinline__ V twiddle24(int j) {
 template <int R, int TWS, typename V>
 __device__ __forceinline__ void dft_regs(V (&v)[R], const V* __restrict__ tw);
 
-// R = 12 or 24 as two R/2-point DFTs of the even and odd elements.
+// R = 12 as two 6-point DFTs of the even and odd elements.
 template <int R, typename V>
 __device__ __forceinline__ void dft_halves(V (&v)[R], const V* __restrict__ tw) {
   V e[R / 2], o[R / 2];
@@ -187,7 +187,7 @@ __device__ __forceinline__ void dft_regs(V (&v)[R], const V* __restrict__ tw) {
     v[4] = csub(e1, t1);
     v[2] = cadd(e2, t2);
     v[5] = csub(e2, t2);
-  } else if constexpr (R == 12 || R == 24) {
+  } else if constexpr (R == 12) {
     dft_halves<R>(v, tw);
   } else {
     dft_regs_pow2<R>(v);

@@ -364,8 +364,7 @@ __global__ void __launch_bounds__(XGeom<T, N>::THREADS, XGeom<T, N>::MIN_BLOCKS)
       inv = (T)1 / (T)n2;
       if (!kp.local_only) ikb = (T)1 / (kc<T>(kp.kbar_fac * 2.0 * M_PI / kp.box, kp.kbkf_f) * sqrt((T)n2));
     }
-    // the Hessian outputs use 1 / (|n|^2 N^3) directly
-    s_inv[k2 * NT + threadIdx.x] = OP == XOP_HESSIAN ? inv * inv_m : inv;
+    s_inv[k2 * NT + threadIdx.x] = inv;
     s_ikb[k2 * NT + threadIdx.x] = ikb;
   }
 
@@ -648,56 +647,25 @@ __global__ void __launch_bounds__(XGeom<T, N>::THREADS, XGeom<T, N>::MIN_BLOCKS)
     return;
   }
 
-  int nout;
-  if (OP == XOP_SOURCE) nout = 1;
-  else if (OP == XOP_SOURCE_LIN || OP == XOP_SHELL) nout = 2;
-  else nout = 4;
-  for (int o = 0; o < nout; ++o) {
-    if (OP == XOP_PHI_FORCE && !((args.nout_mask >> o) & 1)) continue;
+  // XOP_SOURCE, XOP_SOURCE_LIN, XOP_SHELL
+  constexpr int NOUT = OP == XOP_SOURCE ? 1 : 2;
+  for (int o = 0; o < NOUT; ++o) {
     V Y[N2];
 #pragma unroll
     for (int k2 = 0; k2 < N2; ++k2) {
-      const int kx = lane + N1 * k2;
-      const int nx = signed_index(kx, N);
-      const bool nyq_x = kx == N / 2;
+      const int nx = signed_index(lane + N1 * k2, N);
       const int n2 = nx * nx + ny * ny + nz * nz;
       V r = cmake<V>((T)0, (T)0);
       if (n2 != 0) {
-        const T inv_n2 = s_inv[k2 * NT + threadIdx.x];
-        // 1 / kbar = 1 / (kbar_fac * kf * |n|)
-        const T ikb = s_ikb[k2 * NT + threadIdx.x];
-        if (OP == XOP_SOURCE || OP == XOP_SOURCE_LIN) {
+        if (OP == XOP_SHELL) {
+          if (n2 >= args.shell_lo && n2 < args.shell_hi)
+            r = (o == 0) ? cscale(X0[k2], inv_m) : cmake<V>(inv_m, (T)0);
+        } else {
+          // 1 / kbar = 1 / (kbar_fac * kf * |n|)
+          const T ikb = s_ikb[k2 * NT + threadIdx.x];
           const T sfac = kc<T>(kp.s, kp.s_f) * ((T)1 - kc<T>(kp.beta, kp.beta_f) * ikb) * inv_m;
           r = cscale(X0[k2], sfac);
           if (o == 1) r = cscale(r, (T)1 / (kc<T>(kp.alpha, kp.alpha_f) - kc<T>(kp.c2, kp.c2_f) * ikb));
-        } else if (OP == XOP_SHELL) {
-          if (n2 >= args.shell_lo && n2 < args.shell_hi)
-            r = (o == 0) ? cscale(X0[k2], inv_m) : cmake<V>(inv_m, (T)0);
-        } else {  // XOP_PHI_FORCE
-          const T kmag = kf * sqrt((T)n2);
-          const T pref = -kc<T>(kp.aE * kp.aE, kp.aE2_f) / (kmag * kmag);
-          const T om15 = kc<T>(1.5 * (kp.eta - 1.0) / kp.eta, kp.om15_f);
-          V phi;
-          if (kp.gravity == 0) {
-            const T cd = -kc<T>(0.5 / kp.eta, kp.half_inv_eta_f) + kc<T>(kp.c3, kp.c3_f) * ikb;
-            const T den = (T)1 + ikb * kc<T>(1.0 / kp.eta, kp.inv_eta_f);
-            const V rhs = cadd(cscale(X0[k2], om15), cscale(X1[k2], cd));
-            phi = cscale(rhs, pref / den);
-          } else if (kp.gravity == 1) {
-            phi = cscale(X0[k2], pref * om15 * (T)geff_dev(kp, (double)kmag));
-          } else {
-            phi = cscale(X0[k2], pref * om15);
-          }
-          phi = cscale(phi, inv_m);
-          if (o == 0) {
-            r = phi;
-          } else {
-            const int ni = o == 1 ? nx : (o == 2 ? ny : nz);
-            const bool nyq = o == 1 ? nyq_x : (o == 2 ? nyq_y : nyq_z);
-            const T ki = kf * (T)ni;
-            // g = -grad phi -> -i k_i phi
-            r = nyq ? cmake<V>((T)0, (T)0) : cmake<V>(ki * phi.y, -ki * phi.x);
-          }
         }
       }
       Y[k2] = r;
@@ -721,7 +689,7 @@ template <int N> struct XSGeom {
   static constexpr int THREADS = TY * N1;
   static constexpr int TILE = N * TY;  // complex
   static constexpr size_t SMEM = sizeof(float2) * ((size_t)N + 2 * (size_t)TILE);  // phase table, two tiles
-      // REG: the spectrum and the thread's phases W^{q m} stay in registers (two CTAs of 126 registers at
+  // REG: the spectrum and the thread's phases W^{q m} stay in registers (two CTAs of 126 registers at
   // 256^3) instead of being read from shared memory for every output; half the shared-memory
   // instructions, which are what the pass waits for: 75 -> 67.5 us.  At 128^3 the tile version in 64
   // registers lets all 520 CTAs run at once (15.9 us against 17.6 with REG, 17.8 with three per SM).

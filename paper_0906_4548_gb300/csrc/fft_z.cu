@@ -295,7 +295,7 @@ template <typename T, int N> struct AZGeom {
   static constexpr int TY = sizeof(T) == 4 ? 16 : 8;
   static constexpr int THREADS = TY * N1;
   static constexpr int RS0 = N1 * (N2 + 1);
-  static constexpr int RS = N2 < N1 ? RS0 + ((N2 - RS0 % 16) % 16 + 16) % 16 : RS0;  // see relax_rows
+  static constexpr int RS = N2 < N1 ? RS0 + ((N2 - RS0 % 16) % 16 + 16) % 16 : RS0;  // see y_hessian.cu
   static constexpr size_t SMEM = sizeof(vec2_t<T>) * (N + TY * RS + (size_t)N * (TY + 1));
 };
 template <typename T> struct AdjZArgs {

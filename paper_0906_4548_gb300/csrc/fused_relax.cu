@@ -2,13 +2,13 @@
 // FP32 mesh data take relax_tma.cu.
 //
 // A CTA owns TY consecutive rows (x, y0..y0+TY-1) of the mesh.  It
-//   1. inverse-transforms along z the six y-inverted spectra H_xx, H_yy, H_xy,
-//      H_xz, H_yz, N of those rows, two fields of the same row packed into one
+//   1. inverse-transforms along z the six y-inverted spectra a, b, H_xy,
+//      H_xz, H_yz, N of those rows (a, b any two of H_xx, H_yy, H_zz), two fields of the same row packed into one
 //      complex pencil (A + i B: three transforms per row), and folds them into
 //      per-point accumulators held in registers:
 //        q = H_xy^2 + H_xz^2 + H_yz^2 + a^2 + a b + b^2 - (a + b) d,
-//      (a = H_xx, b = H_yy, d the mean-free D; this is
-//      sum_{i<j} (H_ij^2 - H_ii H_jj) with H_zz = d - a - b eliminated), then
+//      (d the mean-free D; this is sum_{i<j} (H_ij^2 - H_ii H_jj) with the
+//      third diagonal one, d - a - b, eliminated), then
 //        R = alpha d - 2 q + c2 N - S                    (Eq. FullDGP2, LHS - RHS)
 //        B' = (1 - w) d^2 + alpha d - R                  (Eq. Bwpara)
 //        Delta = alpha^2 + 4 (1 - w) B', bad points take Delta = 0 (Sec. III.C)
@@ -90,7 +90,7 @@ template <typename T, int N> struct FGeom {
 };
 
 template <typename T> struct FusedArgs {
-  const vec2_t<T>* spec[6];  // y-inverted spectra of H_xx, H_yy, H_xy, H_xz, H_yz, N
+  const vec2_t<T>* spec[6];  // y-inverted spectra of a, b, H_xy, H_xz, H_yz, N
   const T* D;                // current iterate (its mean = dsum / N^3)
   const double* dsum;
   const T* S;                // source field
@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(FGeom<T, N>::THREADS, 2)
   const int lane = threadIdx.x % N1, row = threadIdx.x / N1;
   const int64_t rbase = ((int64_t)x * N + y0 + row) * N;
   const RelaxParams& rp = args.rp;
-  // pairs (H_xx, H_yy) -> G0 and (H_xy, H_xz) -> G1 start loading now
+  // pairs (a, b) -> G0 and (H_xy, H_xz) -> G1 start loading now
   issue_pair<T, N>(args.spec[0], args.spec[1], x, y0, G0);
   issue_pair<T, N>(args.spec[2], args.spec[3], x, y0, G1);
   load_twiddles(s_tw, g_tw, N);
@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(FGeom<T, N>::THREADS, 2)
     if (pr == 0) issue_pair<T, N>(args.spec[4], args.spec[5], x, y0, G0);
     if (pr == 1) issue_source<T, N>(args.S, ((int64_t)x * N + y0) * N, reinterpret_cast<T*>(G1) + TY * N);
     if (pr == 0) {
-      // a = H_xx, b = H_yy:  q = a^2 + a b + b^2 - (a + b) d
+      // q = a^2 + a b + b^2 - (a + b) d
 #pragma unroll
       for (int k2 = 0; k2 < N2; ++k2) {
         AR::q_add_sq(q[k2], ra[k2], ra[k2]);

@@ -59,9 +59,9 @@ enum XOp { XOP_HESSIAN = 0, XOP_SOURCE = 1, XOP_SOURCE_LIN = 2, XOP_PHI_FORCE = 
 // whole grid returns at once (iterations enqueued past the solver's stop).
 // threads: 128, 256 or 512 per CTA (threads / N1 rows per CTA).
 // ctl (may be null): one extra CTA of the launch sums the relaxation's block
-// partials and applies the stop rules, as launch_finalize_control does (the
-// y pass that follows the relaxation pass carries them, one launch fewer per
-// iteration).
+// partials into stats = [sum |R|, sum D_new, bad points, non-finite R] and applies
+// the stop rules (the y pass that follows the relaxation pass carries them, one
+// launch fewer per iteration); abs_src_sum: sum |S| (read at the first iteration).
 struct SolveCtl;
 struct YControl {
   const double* partials;
@@ -160,8 +160,8 @@ struct RelaxParams {
 };
 
 // Fused z pass of a relaxation iteration for FP64 mesh data (fused_relax.cu):
-// inverse z transform of the six y-inverted spectra (H_xx, H_yy, H_xy, H_xz,
-// H_yz, N), residual and update (FP64), forward z transform of D_new into
+// inverse z transform of the six y-inverted spectra (two of H_xx, H_yy, H_zz,
+// then H_xy, H_xz, H_yz, N), residual and update (FP64), forward z transform of D_new into
 // Snew; partials: fused_relax_blocks() x 4 doubles.  arith selects the
 // arithmetic of FP32 mesh data and is not read here (FP32 data take
 // launch_relax_tma below).
@@ -173,7 +173,7 @@ void launch_fused_relax(int arith, vec2_t<T>* const* spec6, const T* D, const do
 template <typename T, int N> int fused_relax_blocks();
 
 // The same pass for FP32 mesh data with TMA tile loads (relax_tma.cu): one
-// tensor map per y-inverted spectrum (H_xx, H_yy, H_xy, H_xz, H_yz, N), built
+// tensor map per y-inverted spectrum (in the same order), built
 // once per context by relax_maps (nonzero when the driver cannot encode them).
 // Every wait inside is bounded by wait_ns; a wait that gives up sets *fault
 // to 1 and its CTA returns.  withhold (a test hook) leaves the first pair's
@@ -186,12 +186,11 @@ struct RelaxMaps {
 // Arguments of one realisation's relaxation pass (relax_tma.cu).
 struct RelaxTmaArgs {
   CUtensorMap map[6];   // y-inverted spectra: two of H_xx, H_yy, H_zz, then H_xy, H_xz, H_yz, N
-  CUtensorMap out_map;  // Snew, for the passes that store it as tiles
+  CUtensorMap out_map;  // z-transformed next iterate, layout S[kz][x][y]
   const float* D;       // current iterate (its mean = dsum / N^3)
   const double* dsum;
   const float* S;       // source field
   float* Dnew;          // next iterate
-  float2* Snew;         // z-transformed next iterate, layout S[kz][x][y]
   double* partials;     // [blocks][4]
   RelaxParams rp;
   const int* skip;
@@ -230,7 +229,7 @@ void launch_y_hessian(const YHessArgs<T>* a, int count, const vec2_t<T>* tw, cud
 
 // Plane-resident Hessian pass (plane.cu) for count <= kBatchMax realisations of one mesh size
 // n (FP32 data; plane_hessian_supported(n)): from the z spectrum in (layout S[kz][x][y]) of
-// each realisation, the six relaxation inputs H_xx, H_yy, H_xy, H_xz, H_yz, N transformed back
+// each realisation, the six relaxation inputs H_yy, H_zz, H_xy, H_xz, H_yz, N transformed back
 // along x and y, in out.p[0..5] (same layout).  Replaces the y pass of the iterate, the Hessian
 // x pass and the six-field inverse y pass of an iteration.  skip as for the other passes.
 struct PlaneArgs {
@@ -317,12 +316,6 @@ struct VerdictBatch {
 };
 void launch_clear_verdicts(const VerdictBatch& b, int count, cudaStream_t s);
 void launch_fetch_verdicts(const VerdictBatch& b, int count, int iters, cudaStream_t s);
-// stats: [sum |R|, sum D_new, bad points, non-finite R] of the iteration
-// it = ctl->next_it (counted on the device, so the same launch serves every
-// iteration of a captured graph); abs_src_sum: sum |S| (read at it = 0);
-// hist[it] receives <|R|> / rnorm.
-void launch_relax_control(SolveCtl* ctl, const double* stats, const double* abs_src_sum, double* hist,
-                          int max_iter, int patience, double tol, double inv_m, cudaStream_t s);
 
 template <typename T>
 void launch_sum(const T* a, int64_t m, bool absval, double* partials, int nblocks, cudaStream_t s);

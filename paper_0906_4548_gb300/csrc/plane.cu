@@ -2,7 +2,7 @@
 //
 // One CTA owns one kz plane of one realisation.  It reads the plane of the z spectrum of
 // the iterate D (layout S[kz][x][y]) once, transforms it forward along y and along x in
-// shared memory, and for each of the six outputs of the relaxation (H_xx, H_yy, H_xy, H_xz,
+// shared memory, and for each of the six outputs of the relaxation (H_yy, H_zz, H_xy, H_xz,
 // H_yz and N, Sec. III.B: nabla_ij C(k) = -k_i k_j C(k), sqrt(-lapbar) C = -D / kbar)
 // forms the multiplier, transforms back along x and y and writes the plane of the output
 // (kz, x, y), ready for the relaxation pass's inverse z transform.  The y and z wavenumbers commute

@@ -195,46 +195,6 @@ void launch_fetch_verdicts(const VerdictBatch& b, int count, int iters, cudaStre
   k_fetch_verdicts<<<count, 128, 0, s>>>(b, iters);
 }
 
-// The stop rules as a launch of their own (relax_control.cuh).
-__global__ void k_relax_control(SolveCtl* __restrict__ c, const double* __restrict__ stats,
-                                const double* __restrict__ abs_src_sum, double* __restrict__ hist,
-                                int max_iter, int patience, double tol, double inv_m) {
-  if (threadIdx.x != 0) return;
-  relax_control_step(c, stats, abs_src_sum, hist, max_iter, patience, tol, inv_m);
-}
-
-void launch_relax_control(SolveCtl* ctl, const double* stats, const double* abs_src_sum, double* hist,
-                          int max_iter, int patience, double tol, double inv_m, cudaStream_t s) {
-  k_relax_control<<<1, 32, 0, s>>>(ctl, stats, abs_src_sum, hist, max_iter, patience, tol, inv_m);
-}
-
-__global__ void __launch_bounds__(256)
-    k_finalize_control(const double* __restrict__ partials, int nblocks, double* __restrict__ stats,
-                       SolveCtl* __restrict__ c, const double* __restrict__ abs_src_sum, double* __restrict__ hist,
-                       int max_iter, int patience, double tol, double inv_m, const int* __restrict__ skip) {
-  if (skip && *skip) return;
-  double v[4] = {0.0, 0.0, 0.0, 0.0};
-  for (int b = threadIdx.x; b < nblocks; b += blockDim.x) {
-    const double4_32a p = reinterpret_cast<const double4_32a*>(partials)[b];
-    v[0] += p.x;
-    v[1] += p.y;
-    v[2] += p.z;
-    v[3] += p.w;
-  }
-  block_sum<4>(v);
-  if (threadIdx.x == 0) {
-    for (int k = 0; k < 4; ++k) stats[k] = v[k];
-    relax_control_step(c, stats, abs_src_sum, hist, max_iter, patience, tol, inv_m);
-  }
-}
-
-void launch_finalize_control(const double* partials, int nblocks, double* stats, SolveCtl* ctl,
-                             const double* abs_src_sum, double* hist, int max_iter, int patience, double tol,
-                             double inv_m, cudaStream_t s, const int* skip) {
-  k_finalize_control<<<1, 256, 0, s>>>(partials, nblocks, stats, ctl, abs_src_sum, hist, max_iter, patience, tol,
-                                       inv_m, skip);
-}
-
 // Per-thread sums of FP32 data run on the FP32 pipe as an unevaluated pair:
 // Knuth's TwoSum keeps every rounding error of the running sum s in c, so
 // s + c is the thread's sum to about 2^-44 relative; the cross-thread and

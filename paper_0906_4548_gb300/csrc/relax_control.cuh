@@ -65,12 +65,4 @@ __device__ __forceinline__ void relax_control_step(SolveCtl* __restrict__ c, con
   c->prev_nbad = nbad;
 }
 
-// One CTA: the fixed-order FP64 sum of the fused relaxation's [nblocks][4]
-// block partials into stats[0..3] (as launch_finalize), then the stop rules
-// above applied to them by thread 0 (the finalize and controller launches of
-// an iteration in one).  skip: as launch_finalize.
-void launch_finalize_control(const double* partials, int nblocks, double* stats, SolveCtl* ctl,
-                             const double* abs_src_sum, double* hist, int max_iter, int patience, double tol,
-                             double inv_m, cudaStream_t s, const int* skip);
-
 }  // namespace dgp

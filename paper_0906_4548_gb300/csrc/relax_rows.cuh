@@ -14,8 +14,8 @@
 // issue (about 63 % of the cycles) and the wait for a CTA's first tiles at 24 warps per SM.  Tried: CTAs
 // that stay and take every gridDim-th tile, loading the next tile's first pair during the forward
 // transform (153 us: the state carried from tile to tile spills at 80 registers, and two CTAs of 128
-// are no faster); two CTAs of 128 registers (159 us).  512^3 holds one CTA of 8 warps and 227
-// registers per SM.
+// are no faster); two CTAs of 128 registers (159 us).  512^3 holds one CTA of 8 warps per SM, of 227
+// registers a thread (168 with pair arithmetic).
 #pragma once
 
 #include "tile_slots.cuh"
@@ -246,7 +246,8 @@ __device__ __forceinline__ void row_forward(unsigned char* buf, const float2* s_
     }
   }
   __syncwarp();
-  // columns k1 = 0 .. N1 / 2: one round, and for Q > 1 a second that holds only k1 = N1 / 2
+  // columns k1 = 0 .. N1 / 2: one round, and a second for those from N2 on (k1 = N1 / 2 alone where
+  // N1 = 2 N2, k1 = 4 .. 6 at 48 = 12 x 4)
   constexpr int ROUNDS = (N1 / 2) / N2 + 1;
   float2 u[ROUNDS][N2];
 #pragma unroll

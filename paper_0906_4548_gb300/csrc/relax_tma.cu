@@ -4,13 +4,13 @@
 // A CTA owns TY = 16 consecutive rows (x, y0 .. y0 + 15) of the mesh.  It
 //   1. inverse-transforms along z the six y-inverted spectra of those rows as
 //      three field pairs (two real fields per complex pencil), in the order
-//        A = (H_xy, H_xz),  B = (H_yz, N),  C = (H_xx, H_yy),
+//        A = (H_xy, H_xz),  B = (H_yz, N),  C = (a, b), two of H_xx, H_yy, H_zz,
 //      and folds them into one accumulator per point,
 //        after A and B:  r = -2 (H_xy^2 + H_xz^2 + H_yz^2) + c2 N,
-//      then with a = H_xx, b = H_yy, the mean-free d = D - <D>, u = a + b and
-//      H_zz = d - u (the trace identity):
-//        R  = r + 2 a b + 2 u H_zz + alpha d - S            (Eq. FullDGP2, LHS - RHS)
-//      (-2 sum_{i<j} (H_ij^2 - H_ii H_jj) = -2 (H_xy^2 + H_xz^2 + H_yz^2) + 2 a b + 2 u H_zz);
+//      then with the mean-free d = D - <D>, u = a + b and the third diagonal one, d - u (the trace
+//      identity):
+//        R  = r + 2 a b + 2 u (d - u) + alpha d - S         (Eq. FullDGP2, LHS - RHS)
+//      (-2 sum_{i<j} (H_ij^2 - H_ii H_jj) = -2 (H_xy^2 + H_xz^2 + H_yz^2) + 2 a b + 2 u (d - u));
 //        B' = d ((1 - w) d + alpha) - R                     (Eq. Bwpara)
 //        Delta = (alpha + 2 (1 - w) d)^2 - 4 (1 - w) R      (= alpha^2 + 4 (1 - w) B')
 //      bad points (Delta < 0) take Delta = 0 (Sec. III.C), and
@@ -85,7 +85,6 @@ struct RxF32 {
     else nonfin += 1.f;
     return o;
   }
-  __device__ static double sum_d(Sum s) { return (double)s; }
 };
 
 // Config-3 mixed arithmetic: R, B' and D_new in FP32 (the FP32 data's own
@@ -118,7 +117,6 @@ struct RxM32 {
     else nonfin += 1.f;
     return o;
   }
-  __device__ static double sum_d(Sum s) { return (double)s; }
 };
 
 struct RxEFT {
@@ -141,7 +139,7 @@ struct RxEFT {
     d.lo -= m_lo;
     d = fp_fast(d.hi, d.lo);
     const FP u = fp_two_sum(a, b);  // a + b exactly
-    FP c = fp_two_sum(d.hi, -u.hi);  // H_zz = d - u
+    FP c = fp_two_sum(d.hi, -u.hi);  // the third diagonal one, d - u
     c.lo += d.lo - u.lo;
     fp_acc(r, fp_prod(2.f * a, b));
     {
@@ -173,7 +171,6 @@ struct RxEFT {
     else nonfin += 1.f;
     return o;
   }
-  __device__ static double sum_d(Sum s) { return (double)s.hi + (double)s.lo; }
 };
 
 // Bound by the FP64 pipe, so r carries half of the sum (factors of two are folded into one FMA at the
@@ -207,7 +204,6 @@ struct RxF64 {
     else nonfin += 1.f;
     return o;
   }
-  __device__ static double sum_d(Sum s) { return s; }
 };
 
 }  // namespace dgp
@@ -258,7 +254,6 @@ int relax_maps(float2* const* spec6, float2* const* snew2, RelaxMaps* out) {
 void relax_set_maps(const RelaxMaps& maps, float2* Snew, RelaxTmaArgs* a) {
   memcpy(a->map, maps.map, sizeof(a->map));
   a->out_map = maps.out_map[Snew == maps.out[0] ? 0 : 1];
-  a->Snew = Snew;
 }
 
 template <int N> int relax_tma_blocks() { return (N / RowGeom<N, false>::TY) * N; }
@@ -301,7 +296,7 @@ void launch_relax_tma_batch(int arith, const RelaxTmaArgs* a, int count, bool of
 }
 
 #define DGP_INST_RT(N)                                                                                          \
-  template int relax_maps<N>(float2* const*, float2* const*, RelaxMaps*);                                                     \
+  template int relax_maps<N>(float2* const*, float2* const*, RelaxMaps*);                                     \
   template int relax_tma_blocks<N>();                                                                         \
   template void launch_relax_tma<N>(int, const RelaxMaps&, const float*, const double*, const float*, float*,  \
                                     float2*, RelaxParams, double*, const float2*, cudaStream_t, const int*, int*, \

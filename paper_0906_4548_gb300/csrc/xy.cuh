@@ -1,4 +1,4 @@
-// The Hessian x pass fused with the six-field inverse y pass (fft_x.cu).
+// The Hessian x pass fused with the inverse y transform of its six outputs (fft_x.cu).
 #pragma once
 
 #include "kernels.cuh"
@@ -7,8 +7,8 @@ namespace dgp {
 
 // FP32 data, N = 128 or 256, one thread-block cluster of N / 16 CTAs per kz plane: from the
 // y-transformed spectrum in (layout S[kz][x][ky]), the six relaxation inputs H_xx, H_yy, H_xy,
-// H_xz, H_yz, N in out.p[0..5], transformed back along x and y (layout S[kz][x][y]), as the
-// Hessian x pass followed by the six-field inverse y pass leaves them.  No-op for other T or N.
+// H_xz, H_yz, N in out.p[0..5], transformed back along x and y (layout S[kz][x][y]); the x pass followed by
+// the Hessian y pass leaves H_yy and H_zz in the first two instead.  No-op for other T or N.
 // skip as for the other passes (read at entry; set by an earlier launch).
 // xy_hessian_available(n): n qualifies and the current device co-schedules the cluster.
 bool xy_hessian_available(int n);
