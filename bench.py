@@ -59,7 +59,7 @@ SORT_EVERY = 8
 NCU_TRAFFIC = {
     "relax": {"bytes": 651.5e6, "sources": ['relax_tma.cu', 'relax_rows.cuh', 'tile_slots.cuh', 'tma.cuh', 'eft.cuh',
                                             'fft_core.cuh', 'kernels.cuh', 'common.cuh'],
-              "sha256": "712b6b3a645c31fb5e9c3bf10a9ae06d9635a6e9eb0733117e6f47a471e75f7c",
+              "sha256": "417342170aaf8b1c9644bb63312369fb4f5cd427e125b9161f71ad4ab5116d2c",
               "profile": "profiles/k_relax_rows_256cube.md"},
 }
 
